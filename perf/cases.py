@@ -288,7 +288,7 @@ def _mlp_params(values, F, K, digits, Y, ranges, seed):
     h = torch.cat([h, torch.ones((len(h), 1), dtype=torch.float64, device="cuda")], 1)
     t = torch.as_tensor(Y / ranges, dtype=torch.float64, device="cuda")
     ridge = 1e-3 * len(h) * torch.eye(h.shape[1], dtype=torch.float64, device="cuda")
-    w = torch.linalg.solve(h.T @ h + ridge, h.T @ t).cpu().numpy()
+    w = np.linalg.solve((h.T @ h + ridge).cpu().numpy(), (h.T @ t).cpu().numpy())
     p["W4"], p["b4"] = w[:-1].T.astype(np.float32), w[-1].astype(np.float32)
     return p
 
