@@ -287,11 +287,12 @@ void launch_mark(uint32_t *evaluated, int64_t ordinal, cudaStream_t st);
 constexpr int kMlpHidden = 256;
 constexpr int kMlpMaxF = 256;           // feature columns (multiple of 16)
 constexpr int kMlpMaxSplits = 64;       // split-K slices of the weight-gradient GEMMs
-// weights of the pipelined forward: chunks of kMlpChunkK K-columns in the
-// shared-memory operand layout, streamed through kMlpStages stages
-constexpr int kMlpChunkK = 32;
-constexpr int kMlpStages = 5;
-constexpr int kMlpStageBytes = kMlpHidden * kMlpChunkK * 2;
+// weights of the fused forward: chunks of kMlpChunkK K-columns in the
+// shared-memory operand layout (the output layer is one chunk); the output
+// layer's rows padded to a multiple of 32 (a pair MMA's N)
+constexpr int kMlpChunkK = 64;
+__host__ __device__ inline int mlp_chunk_k(int l) { return l == 3 ? kMlpHidden : kMlpChunkK; }
+__host__ __device__ inline int mlp_n4(int K) { return (K + 31) & ~31; }
 
 // The network as the fused forward kernel reads it (all device pointers).
 struct MlpDev {
@@ -301,7 +302,7 @@ struct MlpDev {
   const float *range;       // [K] output scale per counter
   const int *off;           // [P + 1] one-hot offset per parameter; off[P] = start of the u block
   const uint16_t *utab;     // [P][16] bf16 u value per digit
-  const uint8_t *wc;        // chunked operand-layout copy of w[0..3] (pipelined forward)
+  const uint8_t *wc;        // chunked operand-layout copy of w[0..3] (fused forward)
   uint32_t wc_off[4];       // byte offset of each layer's first chunk in wc
   uint64_t wait_ns;         // limit of each bounded wait of the forward kernel
   int stall;                // 1: the copy and MMA warps first wait on a barrier nothing arrives at
@@ -367,12 +368,12 @@ void launch_nbr_step(const SearchDev *srch, StepDev *steps_dev, const StepBatch<
                      int num_sms, cudaStream_t st);
 const void *nbr_score_func();
 
-bool mlp_pipe_supported(int F);
-void mlp_pipe_set_attrs();
-void launch_pack_wc(const uint16_t *w, int Nl, int Kl, uint8_t *dst, cudaStream_t st);
-void launch_mlp_pipe(int mode, const MlpDev &md, const uint64_t *packed, int64_t n, float *out,
-                     const float *pcprof, const float *delta, const uint32_t *evaluated,
-                     int *minmax, int *status, int max_ctas, cudaStream_t st);
+// The fused forward on CTA pairs (k_mlp_pair.cu)
+void mlp_pair_set_attrs();
+void launch_pack_wc(const uint16_t *const w[4], int F, int K, int Kp, const uint32_t off[4], uint8_t *dst,
+                    cudaStream_t st);
+void launch_mlp_pair(int mode, const MlpDev &md, const uint64_t *packed, int64_t n, float *out,
+                     const MlpTargets &tg, int *status, int max_ctas, cudaStream_t st);
 void launch_gemm_tc(int epi, const uint16_t *A, int lda, const uint16_t *B, int ldb, int M, int N,
                     int K, const EpiArgs &ep, int *status, cudaStream_t st, int splits = 1);
 // out[M][N] (leading dimension ldo) = the sum, in slice order, of S slices of a

@@ -6,7 +6,7 @@
 //                 of 64; epilogues: FP32 store / bias + GELU (pre-activation,
 //                 bf16 activation and its transpose) / bias / times
 //                 GELU'(pre-activation) (FP32, bf16 and bf16 transpose)
-//   (the fused forward used for predictions and scores is k_mlp_pipe.cu)
+//   (the fused forward used for predictions and scores is k_mlp_pair.cu)
 //   helpers       features of a training batch, transpose, loss gradient,
 //                 column sums, Adam
 //
@@ -32,12 +32,6 @@ __device__ __forceinline__ float gelu_f(float z) {
 __device__ __forceinline__ float gelu_grad_f(float z) {
   return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) +
          z * expf(-0.5f * z * z) * 0.39894228040143268f;
-}
-
-// Order-preserving integer key of a float (for atomicMin / atomicMax).
-__device__ __forceinline__ int okey(float f) {
-  const int b = __float_as_int(f);
-  return b >= 0 ? b : b ^ 0x7FFFFFFF;
 }
 
 __device__ __forceinline__ uint4 pack8(const uint16_t *h) {
@@ -389,7 +383,7 @@ void mlp_set_attrs(int) {
   cudaFuncSetAttribute(k_gemm_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
   cudaFuncSetAttribute(k_gemm_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
   cudaFuncSetAttribute(k_gemm_tc<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
-  mlp_pipe_set_attrs();
+  mlp_pair_set_attrs();
 }
 
 void launch_splitk_sum(const float *ws, int S, size_t stride, int ldw, int M, int N, float *out,
@@ -446,7 +440,7 @@ void launch_to_bf16(const float *p, int rows, int cols, uint16_t *wb, uint16_t *
   k_to_bf16<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p, rows, cols, wb, wt);
 }
 
-// The fused forward (k_mlp_pipe): mode 0 predicted counters, mode 1 Eq. score.
+// The fused forward (k_mlp_pair): mode 0 predicted counters, mode 1 Eq. score.
 void launch_mlp_fwd(int mode, const MlpDev &md, const uint64_t *packed, int64_t n, float *out,
                     const float *pcprof, const float *delta, const uint32_t *evaluated,
                     int *minmax, int *status, int grid, cudaStream_t st) {
@@ -456,7 +450,21 @@ void launch_mlp_fwd(int mode, const MlpDev &md, const uint64_t *packed, int64_t 
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   }
-  launch_mlp_pipe(mode, md, packed, n, out, pcprof, delta, evaluated, minmax, status, sms, st);
+  MlpTargets tg{};
+  if (mode == 1) {
+    tg.S = 1;
+    tg.pcprof[0] = pcprof;
+    tg.delta[0] = delta;
+    tg.s[0] = out;
+    tg.eval[0] = evaluated;
+    tg.mm[0] = minmax;
+  }
+  launch_mlp_pair(mode, md, packed, n, out, tg, status, sms, st);
+}
+
+void launch_mlp_score_shared(const MlpDev &md, const uint64_t *packed, int64_t n,
+                             const MlpTargets &tg, int *status, int max_ctas, cudaStream_t st) {
+  if (tg.S >= 1) launch_mlp_pair(1, md, packed, n, nullptr, tg, status, max_ctas, st);
 }
 
 void launch_mlp_prep(const SearchDev *srch, StepDev *steps_dev, const StepBatch<1> &sb,

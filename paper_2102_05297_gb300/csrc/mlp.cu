@@ -179,8 +179,8 @@ int ensure_pred(ktune_mlp *m, int64_t n) {
 
 // Refresh the chunked weight copy after the bf16 weights changed.
 void pack_weights(ktune_mlp *m) {
-  for (int l = 0; l < 4; ++l)
-    launch_pack_wc(m->d_wb[l], m->rows(2 * l), m->cols(2 * l), m->d_wc + m->wc_off[l], m->stream);
+  const uint16_t *w[4] = {m->d_wb[0], m->d_wb[1], m->d_wb[2], m->d_wb[3]};
+  launch_pack_wc(w, m->F, m->K, m->Kp, m->wc_off, m->d_wc, m->stream);
 }
 
 MlpDev ktune_mlp::dev() const {
@@ -280,11 +280,11 @@ int ktune_mlp_create(ktune_space *s, int K, const int32_t *roles, const float *r
       cudaMemset(m->d_wt[l], 0, n * 2);
     }
   }
-  {  // chunked operand-layout copy of the bf16 weights (pipelined forward)
+  {  // chunked operand-layout copy of the bf16 weights (fused forward)
     uint32_t off = 0;
     for (int l = 0; l < 4; ++l) {
       m->wc_off[l] = off;
-      off += (uint32_t)((size_t)m->rows(2 * l) * m->cols(2 * l) * 2);
+      off += (uint32_t)((l == 3 ? mlp_n4(K) : m->rows(2 * l)) * m->cols(2 * l) * 2);
     }
     if ((rc = dalloc(&m->d_wc, off))) return fail(rc);
     cudaMemset(m->d_wc, 0, off);

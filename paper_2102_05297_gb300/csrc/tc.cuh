@@ -35,6 +35,14 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t
   return d;
 }
 
+// The same from its halves: everything but the start address stays as it is
+// from one K step to the next.
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr, uint32_t lbo) {
+  return ((saddr & 0x3FFFFu) >> 4) | ((lbo >> 4) << 16);
+}
+__device__ __forceinline__ uint32_t sdesc_hi(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }
+__device__ __forceinline__ uint64_t sdesc_of(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
+
 // Instruction descriptor, kind::f16: BF16 A and B (K-major), FP32 D, M x N.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
@@ -90,10 +98,11 @@ __device__ __forceinline__ uint64_t global_ns() {
 }
 
 // Wait for the given phase, giving up after about limit_ns nanoseconds (and
-// after 2^30 polls in any case); returns false if it gave up.
+// after 2^30 polls in any case); returns false if it gave up.  The clock is
+// read only when the first polls fail.
 __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t phase, uint64_t limit_ns) {
   const uint32_t a = smem_u32(mbar);
-  const uint64_t t0 = global_ns();
+  uint64_t t0 = 0;
   for (uint32_t it = 0; it < (1u << 30); ++it) {
     uint32_t done;
     asm volatile(
@@ -102,7 +111,30 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t phase, uint64
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done) : "r"(a), "r"(phase) : "memory");
     if (done) return true;
-    if ((it & 63u) == 63u && global_ns() - t0 > limit_ns) return false;
+    if ((it & 15u) == 15u) {
+      const uint64_t t = global_ns();
+      if (t0 == 0) t0 = t;
+      if (t - t0 > limit_ns) return false;
+    }
+  }
+  return false;
+}
+// The same for waits that are off the critical path: a poll suspends the
+// thread for up to 20 us, so that it leaves the issue slots to others.
+__device__ __forceinline__ bool mbar_wait_idle(uint64_t *mbar, uint32_t phase, uint64_t limit_ns) {
+  const uint32_t a = smem_u32(mbar);
+  uint64_t t0 = 0;
+  for (uint32_t it = 0; it < (1u << 30); ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done) : "r"(a), "r"(phase), "r"(20000u) : "memory");
+    if (done) return true;
+    const uint64_t t = global_ns();
+    if (t0 == 0) t0 = t;
+    if (t - t0 > limit_ns) return false;
   }
   return false;
 }
@@ -121,6 +153,60 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// ---- CTA pairs (cta_group::2): two CTAs of a cluster on one 256-row tile ----
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// All threads of the cluster; shared-memory accesses before it are visible after it.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The address of a shared-memory object of this CTA in the CTA of the given rank.
+__device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t mapped) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(mapped) : "memory");
+}
+__device__ __forceinline__ void tmem_alloc2(uint32_t *dst_smem, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+               :: "r"(smem_u32(dst_smem)), "r"(ncols) : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc2(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" :: "r"(taddr), "r"(ncols)
+               : "memory");
+}
+// D (+)= A * B^T over the pair: A's rows 0..127 and B's first half of the rows
+// come from the even CTA's shared memory, the others from its peer's, at the
+// same offsets; each CTA's tensor memory receives its own 128 rows of D.
+// Issued by one thread of the even CTA.
+__device__ __forceinline__ void mma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
+                                              uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.u32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      :: "r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// Arrive on the mbarrier at this offset in every CTA of the mask once all
+// prior pair MMAs of this thread complete.
+__device__ __forceinline__ void mma_commit_pair(uint64_t *mbar, uint16_t mask) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+      :: "r"(smem_u32(mbar)), "h"(mask) : "memory");
+}
+// One lane of a converged warp, the same one every time.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
 }
 
 __device__ __forceinline__ uint16_t f2bf(float f) {
