@@ -308,20 +308,49 @@ struct MlpDev {
   int stall;                // 1: the copy and MMA warps first wait on a barrier nothing arrives at
 };
 
-// Epilogue operands of the training GEMM (see k_gemm_tc).
-struct EpiArgs {
-  float *c = nullptr;
-  int ldc = 0;
-  const float *bias = nullptr;
-  float *z = nullptr;
-  int ldz = 0;
-  uint16_t *a = nullptr;
-  int lda = 0;
-  uint16_t *at = nullptr;
-  int ldat = 0;
-  size_t split_stride = 0;   // split-K (epilogue 0): slice z of c starts at c + z * split_stride
-  int ntile = 256;           // output columns per CTA (a multiple of 16, at most 256)
+// A training step (k_mlp_train.cu); tensors by layer 0..3, all device pointers.
+struct AdamArgs {
+  float lr, b1, om1, b2, om2, eps, c1, c2;
 };
+struct TrainDev {               // rows: forward, loss gradient, backward
+  int P, F, K, Kp, B;
+  const uint64_t *data;         // packed training configurations
+  const int *idx;               // [B] the batch's rows of data
+  const float *target;          // counters / range, [n][K]
+  const int *off;
+  const uint16_t *utab;
+  const uint16_t *w[4], *wt[4]; // bf16 weights and transposes
+  const float *b[4];
+  uint16_t *xt, *at[3];         // transposes of the layers' inputs: [F][B], [256][B]
+  uint16_t *gzt[3], *gbt;       // transposes of the output gradients: [256][B], [Kp][B]
+  float *gz[3], *g;             // and in float32, [B][256], [B][Kp]
+  double *loss;                 // sum of squared errors, added
+  int *status;
+};
+struct WgradDev {               // weight gradients M x N over B rows, and column sums
+  int B, splits, wg_blocks;
+  const uint16_t *A[4], *X[4];  // [M][B], [N][B]
+  int M[4], N[4], tiles[4];
+  float *ws[4];                 // [splits][M][N]
+  const float *c_src[4];        // [B][c_cols]
+  int c_cols[4];
+  float *c_part[4];             // [row blocks][c_cols]
+  int *status;
+};
+struct UpdateDev {              // tensors W1, b1, W2, b2, W3, b3, W4, b4
+  int rows[8], cols[8];
+  int64_t total;
+  int splits, n_part, adam;
+  const float *ws[4], *part[4];
+  float *g[8], *p[8], *m[8], *v[8];
+  uint16_t *wb[4], *wt[4];
+  AdamArgs a;
+};
+void mlp_train_set_attrs();
+int train_part_rows(int B);     // row blocks of the column sums
+void launch_train_rows(const TrainDev &td, cudaStream_t st);
+void launch_train_wgrad(WgradDev wd, cudaStream_t st);
+void launch_train_update(const UpdateDev &ud, cudaStream_t st);
 
 // The searches one scoring launch of the MLP serves (they share the network
 // and the space): per search its predicted c_profile counters, its Delta, its
@@ -374,25 +403,9 @@ void launch_pack_wc(const uint16_t *const w[4], int F, int K, int Kp, const uint
                     cudaStream_t st);
 void launch_mlp_pair(int mode, const MlpDev &md, const uint64_t *packed, int64_t n, float *out,
                      const MlpTargets &tg, int *status, int max_ctas, cudaStream_t st);
-void launch_gemm_tc(int epi, const uint16_t *A, int lda, const uint16_t *B, int ldb, int M, int N,
-                    int K, const EpiArgs &ep, int *status, cudaStream_t st, int splits = 1);
-// out[M][N] (leading dimension ldo) = the sum, in slice order, of S slices of a
-// split-K workspace (slice z at ws + z * stride, leading dimension ldw).
-void launch_splitk_sum(const float *ws, int S, size_t stride, int ldw, int M, int N, float *out,
-                       int ldo, cudaStream_t st);
-void launch_features(const uint64_t *packed, const int *idx, int B, int P, int F, const int *off,
-                     const uint16_t *utab, uint16_t *X, cudaStream_t st);
-void launch_transpose(const uint16_t *src, int lds, uint16_t *dst, int ldd, int R, int C,
-                      cudaStream_t st);
-void launch_loss_grad(const float *Y, int Kp, const float *T, int K, const int *idx, int B,
-                      float *G, uint16_t *Gb, uint16_t *Gbt, double *loss, cudaStream_t st);
-// column sums of G [R][C] into out [C]; part: scratch of ceil(R / 256) x C floats
-void launch_colsum(const float *G, int R, int C, float *out, float *part, cudaStream_t st);
-struct AdamArgs {
-  float lr, b1, om1, b2, om2, eps, c1, c2;
-};
-void launch_adam(float *p, const float *g, float *m, float *v, int rows, int cols,
-                 const AdamArgs &a, uint16_t *wb, uint16_t *wt, cudaStream_t st);
+// C[M][N] (float32, leading dimension ldc) = A[M][Kd] B[N][Kd]^T
+void launch_gemm_tc(const uint16_t *A, int lda, const uint16_t *B, int ldb, int M, int N, int Kd, float *c,
+                    int ldc, int *status, cudaStream_t st);
 void launch_to_bf16(const float *p, int rows, int cols, uint16_t *wb, uint16_t *wt,
                     cudaStream_t st);
 void launch_mlp_fwd(int mode, const MlpDev &md, const uint64_t *packed, int64_t n, float *out,
@@ -619,16 +632,13 @@ struct ktune_mlp {
   // batch work buffers
   int *d_idx = nullptr;
   int64_t cap_idx = 0;
-  uint16_t *d_X = nullptr, *d_Xt = nullptr;
-  float *d_Z[3] = {};
-  uint16_t *d_A[3] = {}, *d_At[3] = {};
-  float *d_Y = nullptr, *d_G = nullptr;
-  uint16_t *d_Gb = nullptr, *d_Gbt = nullptr;
-  float *d_Gz[2] = {};
-  uint16_t *d_Gzb[2] = {}, *d_Gzbt[2] = {};
+  uint16_t *d_Xt = nullptr, *d_At[3] = {};   // transposes of the layers' inputs
+  float *d_G = nullptr, *d_Gz[3] = {};       // output gradients, float32 and bf16 transposes
+  uint16_t *d_Gbt = nullptr, *d_Gzt[3] = {};
   double *d_loss = nullptr;
   int *d_status = nullptr;
-  float *d_ws = nullptr;                // split-K workspace of the weight gradients
+  float *d_ws = nullptr;                // slices of the weight gradients
+  float *d_part = nullptr;              // row blocks of the bias gradients
   // prediction staging
   uint64_t *d_pred_in = nullptr;
   float *d_pred_out = nullptr;

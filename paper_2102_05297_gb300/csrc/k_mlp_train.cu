@@ -1,0 +1,492 @@
+// One training step of the MLP counter model in three launches.
+//
+//   k_train_rows   everything that is independent per row -- features, the
+//                  three hidden layers, the output layer with the loss and its
+//                  gradient, and the three backward layers -- for 128 rows per
+//                  cluster of four CTAs.  CTA r computes columns [64 r, 64 r + 64)
+//                  of every hidden layer (tcgen05, M = 128, N = 64) and stores
+//                  its bfloat16 activations into all four CTAs' operand buffers
+//                  (distributed shared memory); pre-activations stay in tensor
+//                  memory as accumulators (z = accumulator + bias again in the
+//                  backward pass), so no layer reads or writes memory but for
+//                  the transposes that the weight gradients need;
+//   k_train_wgrad  the four weight gradients, whose reduction runs over the
+//                  batch, split over up to 64 slices of rows, each slice's tile
+//                  into a workspace, and the bias gradients' row-block sums;
+//   k_train_update the slices summed in a fixed order, and Adam.
+// What bounds it: latency.  The step's arithmetic is 0.4 GFLOP x 9 (about 2 us of
+// tensor work at 4,096 rows); k_train_rows is a chain of seven layers, each an
+// MMA, an epilogue of erff / expf and a cluster barrier.  As 38 launches (one
+// GEMM per layer and direction, transposes, sums and one Adam per tensor) a
+// step took 299 us.
+// Every wait on the tensor cores is bounded: on time-out the kernels record
+// KTUNE_ETIMEOUT, wait once more (bounded) for their MMAs in flight and go on
+// to their end with whatever was computed.
+#include <float.h>
+#include <limits.h>
+
+#include <algorithm>
+
+#include "device_common.cuh"
+#include "internal.h"
+#include "tc.cuh"
+
+namespace ktune {
+
+namespace {
+
+constexpr uint64_t kTrainWait = 1000000000ull;   // 1 s per tensor-core wait
+constexpr int kRows = 128;                       // rows per cluster
+constexpr int kSplitN = 4;                       // CTAs per cluster
+constexpr int kCols = kMlpHidden / kSplitN;      // hidden columns per CTA
+constexpr int kRowThreads = 512;
+constexpr int kActBuf = kRows * kMlpHidden * 2;  // 64 KB
+constexpr int kWBuf = kCols * kMlpHidden * 2;    // 32 KB: 64 x 256 (or K x 256 of the output layer)
+constexpr int kRowSmem = 2 * kActBuf + 2 * kWBuf;
+
+__device__ __forceinline__ float gelu_f(float z) {
+  return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f));
+}
+__device__ __forceinline__ float gelu_grad_f(float z) {
+  return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) +
+         z * expf(-0.5f * z * z) * 0.39894228040143268f;
+}
+
+// Rows x Kd bf16 (row-major, leading dimension ld) into core matrices with KC = Kd.
+__device__ __forceinline__ void load_rows(uint8_t *dst, const uint16_t *src, int ld, int rows, int Kd) {
+  const int per_row = Kd >> 3, pieces = rows * per_row;
+  for (int p = threadIdx.x; p < pieces; p += blockDim.x) {
+    const int r = p / per_row, kb = p - r * per_row;
+    cp_async16(dst + tc::core_off(r, kb * 8, Kd), src + (size_t)r * ld + kb * 8);
+  }
+}
+
+__device__ __forceinline__ uint4 pack8(const uint16_t *h) {
+  uint4 q;
+  q.x = h[0] | ((uint32_t)h[1] << 16);
+  q.y = h[2] | ((uint32_t)h[3] << 16);
+  q.z = h[4] | ((uint32_t)h[5] << 16);
+  q.w = h[6] | ((uint32_t)h[7] << 16);
+  return q;
+}
+
+__device__ __forceinline__ void st_cluster16(uint32_t addr, const uint4 &v) {
+  asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y),
+               "r"(v.z), "r"(v.w)
+               : "memory");
+}
+
+__global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1)
+    k_train_rows(const __grid_constant__ TrainDev td) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  __shared__ uint64_t mbar;
+  __shared__ uint32_t tmem_base;
+  __shared__ float sh_b[3][kCols], sh_b4[KTUNE_MAX_COUNTERS];
+  __shared__ uint8_t sh_col[kMlpMaxF];             // the parameter of a feature column
+  __shared__ uint16_t sh_utab[KTUNE_MAX_PARAMS * 16];
+  __shared__ int sh_off[KTUNE_MAX_PARAMS + 1];
+  uint8_t *const act[2] = {sm, sm + kActBuf};
+  uint8_t *const wb[2] = {sm + 2 * kActBuf, sm + 2 * kActBuf + kWBuf};
+  const int F = td.F, K = td.K, Kp = td.Kp, B = td.B, H = kMlpHidden;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = (int)tc::cluster_rank(), n0 = rank * kCols;
+  const int row = (warp & 3) * 32 + lane, chunk = 16 * (warp >> 2);   // this thread's row and columns
+  const int b = (int)(blockIdx.x / kSplitN) * kRows + row;            // its batch row
+  const bool live = b < B;
+  bool ok = true;
+  uint32_t phase = 0;
+
+  // weights of the first two layers on their way
+  load_rows(wb[0], td.w[0] + (size_t)n0 * F, F, kCols, F);
+  cp_async_commit();
+  load_rows(wb[1], td.w[1] + (size_t)n0 * H, H, kCols, H);
+  cp_async_commit();
+  if (warp == 0) tc::tmem_alloc(&tmem_base, 512);
+  if (threadIdx.x == 0) tc::mbar_init(&mbar, 1);
+  for (int i = threadIdx.x; i < 3 * kCols; i += blockDim.x) sh_b[i / kCols][i % kCols] = td.b[i / kCols][n0 + i % kCols];
+  for (int i = threadIdx.x; i < Kp; i += blockDim.x) sh_b4[i] = td.b[3][i];
+  for (int i = threadIdx.x; i <= td.P; i += blockDim.x) sh_off[i] = td.off[i];
+  for (int i = threadIdx.x; i < td.P * 16; i += blockDim.x) sh_utab[i] = td.utab[i];
+  const int src = live ? td.idx[b] : 0;
+  const uint64_t pk = live ? td.data[src] : 0ull;
+  __syncthreads();
+  for (int c = threadIdx.x; c < F; c += blockDim.x) {
+    int j = 0;
+    while (j + 1 < td.P && sh_off[j + 1] <= c) ++j;
+    sh_col[c] = (uint8_t)(c >= sh_off[td.P] ? min(c - sh_off[td.P], td.P) : j);
+  }
+  __syncthreads();
+  // features: one-hot digits, u per parameter, zeros; four threads per row
+  for (int G = warp >> 2; G < F / 8; G += 4) {
+    uint16_t v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int c = 8 * G + e, j = sh_col[c];
+      uint16_t x = 0;
+      if (live) {
+        if (c >= sh_off[td.P]) x = j < td.P ? sh_utab[j * 16 + nib64(pk, j)] : (uint16_t)0;
+        else x = (int)nib64(pk, j) == c - sh_off[j] ? (uint16_t)0x3F80 : (uint16_t)0;
+      }
+      v[e] = x;
+      // each CTA of the cluster stores a quarter of the transpose
+      if (live && (G & 3) == rank) td.xt[(size_t)c * B + b] = x;
+    }
+    *reinterpret_cast<uint4 *>(act[0] + tc::core_off(row, 8 * G, F)) = pack8(v);
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::cluster_sync();      // every CTA of the cluster runs: its shared memory may be written
+  tc::fence_after();
+  const uint32_t tmem = tmem_base, lanes = (uint32_t)((warp & 3) * 32) << 16;
+
+  // D[dcol ..) = act * w^T over Kd columns; returns when it is complete and the
+  // weights of the layer after the next may be loaded into w's buffer
+  auto layer = [&](const uint8_t *a, const uint8_t *w, int Kd, int N, uint32_t dcol) {
+    cp_async_wait_group<1>();        // this layer's weights (the next layer's may be in flight)
+    tc::fence_async_smem();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      tc::fence_async_smem();        // what the other CTAs stored, behind the cluster barrier
+      tc::fence_after();
+      const uint32_t idesc = tc::idesc_bf16(128, N);
+      const uint32_t hi = tc::sdesc_hi((uint32_t)Kd * 16u);
+      uint32_t al = tc::sdesc_lo(tc::smem_u32(a), 128), wl = tc::sdesc_lo(tc::smem_u32(w), 128);
+      for (int k = 0; k < Kd; k += 16, al += 16, wl += 16)   // 256 bytes per step
+        tc::mma_bf16(tmem + dcol, tc::sdesc_of(al, hi), tc::sdesc_of(wl, hi), idesc, k ? 1u : 0u);
+      tc::mma_commit(&mbar);
+    }
+    bool w_ok = tc::mbar_wait(&mbar, phase, kTrainWait);
+    if (!w_ok) w_ok = tc::mbar_wait(&mbar, phase, kTrainWait) && false;   // the MMAs still in flight
+    ok = ok && w_ok;
+    phase ^= 1u;
+    tc::fence_after();
+  };
+  // 16 bf16 of this thread's row and columns into every CTA's buffer `dst`
+  auto share = [&](uint8_t *dst, const uint16_t (&h)[16]) {
+    const uint4 q0 = pack8(h), q1 = pack8(h + 8);
+    const uint32_t at = tc::smem_u32(dst) + tc::core_off(row, n0 + chunk, H);
+#pragma unroll
+    for (int r = 0; r < kSplitN; ++r) {
+      const uint32_t p = tc::map_rank(at, (uint32_t)r);
+      st_cluster16(p, q0);
+      st_cluster16(p + 128u, q1);
+    }
+  };
+  auto barrier = [&]() {
+    asm volatile("fence.proxy.async;" ::: "memory");
+    tc::fence_before();
+    __syncwarp();
+    tc::cluster_sync();
+    tc::fence_after();
+  };
+
+  // ---- forward: hidden layers 0..2 (accumulators in columns 64 l) ----------------------
+#pragma unroll 1
+  for (int l = 0; l < 3; ++l) {
+    layer(act[l & 1], wb[l & 1], l == 0 ? F : H, kCols, (uint32_t)(l * kCols));
+    if (l == 0) load_rows(wb[0], td.w[2] + (size_t)n0 * H, H, kCols, H);
+    else if (l == 1) load_rows(wb[1], td.w[3], H, Kp, H);
+    else load_rows(wb[0], td.wt[3] + (size_t)n0 * Kp, Kp, kCols, Kp);
+    cp_async_commit();
+    float v[16];
+    uint16_t h[16];
+    tc::tmem_ld16(tmem + lanes + (uint32_t)(l * kCols + chunk), v);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      h[i] = tc::f2bf(gelu_f(__fadd_rn(v[i], sh_b[l][chunk + i])));
+      if (live) td.at[l][(size_t)(n0 + chunk + i) * B + b] = h[i];
+    }
+    share(act[(l + 1) & 1], h);
+    barrier();
+  }
+  // ---- output layer, loss and its gradient (every CTA of the cluster, its own copy) ----
+  {
+    float t[16];
+    const bool mine = chunk < Kp;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      t[i] = live && chunk + i < K ? td.target[(size_t)src * K + chunk + i] : 0.0f;
+    layer(act[1], wb[1], H, Kp, 3u * kCols);
+    load_rows(wb[1], td.wt[2] + (size_t)n0 * H, H, kCols, H);
+    cp_async_commit();
+    double e = 0.0;
+    if (mine) {
+      float v[16], g[16];
+      uint16_t h[16];
+      tc::tmem_ld16(tmem + lanes + (uint32_t)(3 * kCols + chunk), v);
+      const float bk = (float)B * (float)K;      // below 2^24: exact
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        g[i] = 0.0f;
+        if (live && chunk + i < K) {
+          const float d = __fsub_rn(__fadd_rn(v[i], sh_b4[chunk + i]), t[i]);
+          if ((i >> 2) == rank) e += (double)d * (double)d;
+          // 2 d / (B K), one rounding (a float64 quotient rounded to float32 is the same number)
+          g[i] = __fdiv_rn(2.0f * d, bk);
+        }
+        h[i] = tc::f2bf(g[i]);
+        if (live && (i >> 2) == rank) td.gbt[(size_t)(chunk + i) * B + b] = h[i];
+      }
+      if (live)
+#pragma unroll
+        for (int i = 0; i < 16; i += 4)
+          if ((i >> 2) == rank)
+            *reinterpret_cast<float4 *>(td.g + (size_t)b * Kp + chunk + i) =
+                make_float4(g[i], g[i + 1], g[i + 2], g[i + 3]);
+      *reinterpret_cast<uint4 *>(act[0] + tc::core_off(row, chunk, Kp)) = pack8(h);
+      *reinterpret_cast<uint4 *>(act[0] + tc::core_off(row, chunk + 8, Kp)) = pack8(h + 8);
+    }
+    for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (lane == 0 && e != 0.0) atomicAdd(td.loss, e);
+    barrier();               // every CTA's output layer has read its activations
+  }
+  // ---- backward: g_z(l) = (g(l + 1) W(l + 1)) GELU'(z(l)), l = 2, 1, 0 -------------------
+#pragma unroll 1
+  for (int l = 2; l >= 0; --l) {
+    const int s = l & 1;                       // l = 2: act[0], wb[0]; 1: act[1], wb[1]; 0: act[0], wb[0]
+    const uint32_t dcol = 256u + (uint32_t)(l * kCols);
+    layer(act[s], wb[s], l == 2 ? Kp : H, kCols, dcol);
+    if (l == 2) load_rows(wb[0], td.wt[1] + (size_t)n0 * H, H, kCols, H);
+    cp_async_commit();
+    float v[16], z[16];
+    uint16_t h[16];
+    tc::tmem_ld16(tmem + lanes + (uint32_t)(l * kCols + chunk), z);
+    tc::tmem_ld16(tmem + lanes + dcol + (uint32_t)chunk, v);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      v[i] = __fmul_rn(v[i], gelu_grad_f(__fadd_rn(z[i], sh_b[l][chunk + i])));
+      h[i] = tc::f2bf(v[i]);
+      if (live) td.gzt[l][(size_t)(n0 + chunk + i) * B + b] = h[i];
+    }
+    if (live)
+#pragma unroll
+      for (int i = 0; i < 16; i += 4)
+        *reinterpret_cast<float4 *>(td.gz[l] + (size_t)b * H + n0 + chunk + i) =
+            make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    if (l > 0) {
+      share(act[s ^ 1], h);
+      barrier();
+    }
+  }
+  cp_async_wait_all();
+  if (!ok && threadIdx.x == 0) atomicExch(td.status, KTUNE_ETIMEOUT);
+  tc::fence_before();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, 512);
+}
+
+// ---- weight gradients ---------------------------------------------------------------
+constexpr int kWgThreads = 256;
+constexpr int kWgTile = 128;                     // output rows and columns per CTA
+constexpr int kWgStage = 2 * kWgTile * 64 * 2;   // both operands' 64 columns of K
+constexpr int kWgSmem = 2 * kWgStage;            // three CTAs per SM
+constexpr int kColRows = 256;                    // rows per block of the bias gradients' sums
+
+// Rows [0, rows) x columns [k0, k0 + kc) into core matrices with KC = kc by
+// asynchronous copies; rows >= valid are 0.
+__device__ __forceinline__ void load_tile(uint8_t *dst, const uint16_t *src, int ld, int rows, int valid,
+                                          int k0, int kc) {
+  const int per_row = kc >> 3, pieces = rows * per_row;
+  for (int p = threadIdx.x; p < pieces; p += blockDim.x) {
+    const int r = p / per_row, kb = p - r * per_row;
+    uint8_t *d = dst + tc::core_off(r, kb * 8, kc);
+    if (r < valid) cp_async16(d, src + (size_t)r * ld + k0 + kb * 8);
+    else *reinterpret_cast<uint4 *>(d) = make_uint4(0, 0, 0, 0);
+  }
+}
+
+// Blocks below wg_blocks: slice z of one 128 x 128 tile of a weight gradient
+// (G^T X over the slice's rows) into the workspace.  The blocks behind them: one
+// (32 columns, 256 rows) block of a bias gradient, in the order of a 32-row
+// stride: rows y, y + 32, ... per y in float32, then the 32 partials in y order.
+__global__ void __launch_bounds__(kWgThreads) k_train_wgrad(const __grid_constant__ WgradDev wd) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  __shared__ uint64_t mbar;
+  __shared__ uint32_t tmem_base;
+  __shared__ float part[32][33];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int B = wd.B;
+  if ((int)blockIdx.x >= wd.wg_blocks) {
+    int q = (int)blockIdx.x - wd.wg_blocks;
+    const int nb = (B + kColRows - 1) / kColRows;
+    const int rb = q % nb;
+    q /= nb;
+    int t = 0;
+    while (q >= (wd.c_cols[t] + 31) / 32) q -= (wd.c_cols[t++] + 31) / 32;
+    const int C = wd.c_cols[t], c = q * 32 + lane;
+    const int r0 = rb * kColRows, r1 = min(B, r0 + kColRows);
+    for (int y = warp; y < 32; y += kWgThreads / 32) {
+      float s = 0.0f;
+      if (c < C)
+        for (int r = r0 + y; r < r1; r += 32) s = __fadd_rn(s, wd.c_src[t][(size_t)r * C + c]);
+      part[y][lane] = s;
+    }
+    __syncthreads();
+    if (warp == 0 && c < C) {
+      float s = 0.0f;
+      for (int y = 0; y < 32; ++y) s = __fadd_rn(s, part[y][lane]);
+      wd.c_part[t][(size_t)rb * C + c] = s;
+    }
+    return;
+  }
+  int tile = (int)blockIdx.x / wd.splits, p = 0;
+  const int z = (int)blockIdx.x - tile * wd.splits;
+  while (tile >= wd.tiles[p]) tile -= wd.tiles[p++];
+  const int M = wd.M[p], N = wd.N[p], nt = (N + kWgTile - 1) / kWgTile;
+  const int m0 = tile / nt * kWgTile, c0 = tile % nt * kWgTile;
+  const int Nt = min(kWgTile, N - c0), Nm = (Nt + 15) & ~15;
+  const uint16_t *A = wd.A[p] + (size_t)m0 * B, *X = wd.X[p] + (size_t)c0 * B;
+  // this slice's rows, in whole chunks of 64
+  const int n_chunks = (B + 63) / 64;
+  const int lo = (int)((int64_t)n_chunks * z / wd.splits), hi = (int)((int64_t)n_chunks * (z + 1) / wd.splits);
+  if (warp == 0) tc::tmem_alloc(&tmem_base, 128);
+  if (threadIdx.x == 0) tc::mbar_init(&mbar, 1);
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tmem = tmem_base;
+  uint32_t phase = 0;
+  bool ok = true;
+  auto issue = [&](int c) {
+    const int k0 = c * 64, kc = min(64, B - k0);
+    uint8_t *s = sm + (c & 1) * kWgStage;
+    load_tile(s, A, B, kWgTile, M - m0, k0, kc);
+    load_tile(s + kWgStage / 2, X, B, Nm, Nt, k0, kc);
+    cp_async_commit();
+  };
+  auto done = [&]() {
+    bool w = tc::mbar_wait(&mbar, phase, kTrainWait);
+    if (!w) w = tc::mbar_wait(&mbar, phase, kTrainWait) && false;
+    phase ^= 1u;
+    ok = ok && w;
+    tc::fence_after();
+  };
+  if (lo < hi) issue(lo);
+  for (int c = lo; c < hi; ++c) {
+    // the MMAs of chunk c - 1 read the stage that chunk c + 1 is copied into
+    if (c > lo) {
+      done();
+      __syncthreads();
+    }
+    if (c + 1 < hi) {
+      issue(c + 1);
+      cp_async_wait_group<1>();
+    } else {
+      cp_async_wait_group<0>();
+    }
+    tc::fence_async_smem();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      tc::fence_after();
+      const int kc = min(64, B - c * 64);
+      const uint32_t idesc = tc::idesc_bf16(128, Nm), dh = tc::sdesc_hi((uint32_t)kc * 16u);
+      const uint32_t s = tc::smem_u32(sm + (c & 1) * kWgStage);
+      uint32_t al = tc::sdesc_lo(s, 128), xl = tc::sdesc_lo(s + kWgStage / 2, 128);
+      for (int k = 0; k < kc; k += 16, al += 16, xl += 16)
+        tc::mma_bf16(tmem, tc::sdesc_of(al, dh), tc::sdesc_of(xl, dh), idesc, c > lo || k ? 1u : 0u);
+      tc::mma_commit(&mbar);
+    }
+  }
+  if (lo < hi) done();
+  // slices of fewer rows than 64 x splits may be empty: zeros
+  const int row = m0 + (warp & 3) * 32 + lane;
+  float *out = wd.ws[p] + (size_t)z * M * N + (size_t)row * N + c0;
+  for (int c = 16 * (warp >> 2); c < Nt; c += 32) {
+    float v[16];
+    if (lo < hi) {
+      tc::tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + c, v);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] = 0.0f;
+    }
+    if (row < M)
+#pragma unroll
+      for (int i = 0; i < 16; i += 4)
+        *reinterpret_cast<float4 *>(out + c + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+  }
+  if (!ok && threadIdx.x == 0) atomicExch(wd.status, KTUNE_ETIMEOUT);
+  tc::fence_before();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, 128);
+}
+
+// ---- sums over the slices and Adam ----------------------------------------------------
+// One thread per parameter: a weight's slices in order (float32), a bias's row
+// blocks in order (float64), then, if adam, the update (every operation one
+// float32 rounding) with the refreshed bf16 copy and its transpose; otherwise
+// the gradient itself.
+__global__ void __launch_bounds__(256) k_train_update(const __grid_constant__ UpdateDev ud) {
+  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= ud.total) return;
+  int t = 0;
+  while (i >= (int64_t)ud.rows[t] * ud.cols[t]) i -= (int64_t)ud.rows[t] * ud.cols[t], ++t;
+  float gi;
+  if (t & 1) {
+    double s = 0.0;
+    for (int q = 0; q < ud.n_part; ++q) s += (double)ud.part[t >> 1][(size_t)q * ud.cols[t] + i];
+    gi = (float)s;
+  } else {
+    const float *w = ud.ws[t >> 1] + i;
+    const size_t stride = (size_t)ud.rows[t] * ud.cols[t];
+    gi = 0.0f;
+    int z = 0;
+    for (; z + 8 <= ud.splits; z += 8) {       // eight loads in flight, added in order
+      float v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = w[(size_t)(z + e) * stride];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) gi = __fadd_rn(gi, v[e]);
+    }
+    for (; z < ud.splits; ++z) gi = __fadd_rn(gi, w[(size_t)z * stride]);
+  }
+  if (!ud.adam) {
+    ud.g[t][i] = gi;
+    return;
+  }
+  const AdamArgs &a = ud.a;
+  const float mi = __fadd_rn(__fmul_rn(a.b1, ud.m[t][i]), __fmul_rn(a.om1, gi));
+  const float vi = __fadd_rn(__fmul_rn(a.b2, ud.v[t][i]), __fmul_rn(__fmul_rn(a.om2, gi), gi));
+  ud.m[t][i] = mi;
+  ud.v[t][i] = vi;
+  const float mh = __fdiv_rn(mi, a.c1), vh = __fdiv_rn(vi, a.c2);
+  const float pi =
+      __fsub_rn(ud.p[t][i], __fdiv_rn(__fmul_rn(a.lr, mh), __fadd_rn(__fsqrt_rn(vh), a.eps)));
+  ud.p[t][i] = pi;
+  if (t & 1) return;
+  const uint16_t h = tc::f2bf(pi);
+  ud.wb[t >> 1][i] = h;
+  if (ud.wt[t >> 1]) {
+    const int r = (int)(i / ud.cols[t]), c = (int)(i - (int64_t)r * ud.cols[t]);
+    ud.wt[t >> 1][(size_t)c * ud.rows[t] + r] = h;
+  }
+}
+
+}  // namespace
+
+void mlp_train_set_attrs() {
+  cudaFuncSetAttribute(k_train_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem);
+  cudaFuncSetAttribute(k_train_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
+}
+
+void launch_train_rows(const TrainDev &td, cudaStream_t st) {
+  k_train_rows<<<kSplitN * ((td.B + kRows - 1) / kRows), kRowThreads, kRowSmem, st>>>(td);
+}
+
+int train_part_rows(int B) { return (B + kColRows - 1) / kColRows; }
+
+void launch_train_wgrad(WgradDev wd, cudaStream_t st) {
+  int blocks = 0;
+  for (int p = 0; p < 4; ++p) {
+    wd.tiles[p] = ((wd.M[p] + kWgTile - 1) / kWgTile) * ((wd.N[p] + kWgTile - 1) / kWgTile);
+    blocks += wd.tiles[p] * wd.splits;
+  }
+  wd.wg_blocks = blocks;
+  for (int t = 0; t < 4; ++t) blocks += (wd.c_cols[t] + 31) / 32 * train_part_rows(wd.B);
+  k_train_wgrad<<<blocks, kWgThreads, kWgSmem, st>>>(wd);
+}
+
+void launch_train_update(const UpdateDev &ud, cudaStream_t st) {
+  k_train_update<<<(unsigned)((ud.total + 255) / 256), 256, 0, st>>>(ud);
+}
+
+}  // namespace ktune

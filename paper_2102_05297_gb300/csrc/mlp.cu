@@ -1,6 +1,5 @@
 // Host side of the MLP counter model: parameters, training set, the training
-// step (forward, loss gradient, backward, Adam) as a sequence of tensor-core
-// GEMMs, and predictions through the fused forward kernel.
+// step (rows, weight gradients, update: three launches), and predictions through the fused forward kernel.
 #include <math.h>
 #include <string.h>
 
@@ -81,79 +80,76 @@ int upload_idx(ktune_mlp *m, const int32_t *idx, int64_t n) {
   return KTUNE_OK;
 }
 
-// Forward and backward over B rows d_idx[row0 ..]; gradients into d_g, the
-// squared-error sum added to d_loss.
-void enqueue_fwd_bwd(ktune_mlp *m, const int *idx, int B) {
-  cudaStream_t st = m->stream;
-  const int F = m->F, H = kMlpHidden, Kp = m->Kp;
-  int *status = m->d_status;
-  launch_features(m->d_data, idx, B, m->P, F, m->d_off, m->d_utab, m->d_X, st);
-  launch_transpose(m->d_X, F, m->d_Xt, B, B, F, st);
-  const uint16_t *a_prev = m->d_X;
-  int lda_prev = F;
+int train_splits(int B) { return std::min(kMlpMaxSplits, std::max(1, (B + 127) / 128)); }
+
+// Forward and backward over the B rows idx, the squared-error sum added to
+// *loss, then the gradients into d_g (adam null) or the Adam update.
+void enqueue_step(ktune_mlp *m, const int *idx, int B, double *loss, const AdamArgs *adam) {
+  const int H = kMlpHidden;
+  TrainDev td{};
+  td.P = m->P;
+  td.F = m->F;
+  td.K = m->K;
+  td.Kp = m->Kp;
+  td.B = B;
+  td.data = m->d_data;
+  td.idx = idx;
+  td.target = m->d_target;
+  td.off = m->d_off;
+  td.utab = m->d_utab;
+  for (int l = 0; l < 4; ++l) {
+    td.w[l] = m->d_wb[l];
+    td.wt[l] = m->d_wt[l];
+    td.b[l] = m->d_p[2 * l + 1];
+  }
+  td.xt = m->d_Xt;
   for (int l = 0; l < 3; ++l) {
-    EpiArgs e;
-    e.bias = m->d_p[2 * l + 1];
-    e.z = m->d_Z[l];
-    e.ldz = H;
-    e.a = m->d_A[l];
-    e.lda = H;
-    e.at = m->d_At[l];
-    e.ldat = B;
-    e.ntile = 64;   // 4 x more CTAs: the epilogue (GELU of every element) dominates
-    launch_gemm_tc(1, a_prev, lda_prev, m->d_wb[l], l == 0 ? F : H, B, H, l == 0 ? F : H, e,
-                   status, st);
-    a_prev = m->d_A[l];
-    lda_prev = H;
+    td.at[l] = m->d_At[l];
+    td.gzt[l] = m->d_Gzt[l];
+    td.gz[l] = m->d_Gz[l];
   }
-  {
-    EpiArgs e;
-    e.c = m->d_Y;
-    e.ldc = Kp;
-    e.bias = m->d_p[7];
-    launch_gemm_tc(2, m->d_A[2], H, m->d_wb[3], H, B, Kp, H, e, status, st);
+  td.gbt = m->d_Gbt;
+  td.g = m->d_G;
+  td.loss = loss;
+  td.status = m->d_status;
+  launch_train_rows(td, m->stream);
+
+  WgradDev wd{};
+  UpdateDev ud{};
+  wd.B = B;
+  wd.splits = ud.splits = train_splits(B);
+  wd.status = m->d_status;
+  ud.n_part = train_part_rows(B);
+  float *ws = m->d_ws, *part = m->d_part;
+  for (int l = 0; l < 4; ++l) {
+    wd.A[l] = l == 3 ? m->d_Gbt : m->d_Gzt[l];
+    wd.X[l] = l == 0 ? m->d_Xt : m->d_At[l - 1];
+    wd.M[l] = m->rows(2 * l);
+    wd.N[l] = m->cols(2 * l);
+    wd.ws[l] = ws;
+    ws += (size_t)wd.splits * wd.M[l] * wd.N[l];
+    wd.c_src[l] = l == 3 ? m->d_G : m->d_Gz[l];
+    wd.c_cols[l] = l == 3 ? m->Kp : H;
+    wd.c_part[l] = part;
+    part += (size_t)ud.n_part * wd.c_cols[l];
+    ud.ws[l] = wd.ws[l];
+    ud.part[l] = wd.c_part[l];
+    ud.wb[l] = m->d_wb[l];
+    ud.wt[l] = m->d_wt[l];
   }
-  launch_loss_grad(m->d_Y, Kp, m->d_target, m->K, idx, B, m->d_G, m->d_Gb, m->d_Gbt, m->d_loss,
-                   st);
-  // weight gradients: K is the batch, split over up to 64 CTA groups, the
-  // slices summed in a fixed order
-  const int splits = std::min(kMlpMaxSplits, std::max(1, (B + 127) / 128));
-  auto wgrad = [&](const uint16_t *gt, const uint16_t *xt, int M, int N, float *out) {
-    EpiArgs e;
-    e.c = m->d_ws;
-    e.ldc = N;
-    e.split_stride = (size_t)M * N;
-    launch_gemm_tc(0, gt, B, xt, B, M, N, B, e, status, st, splits);
-    launch_splitk_sum(m->d_ws, splits, (size_t)M * N, N, M, N, out, N, st);
-  };
-  // layer 4
-  launch_colsum(m->d_G, B, Kp, m->d_g[7], m->d_ws, st);
-  wgrad(m->d_Gbt, m->d_At[2], Kp, H, m->d_g[6]);
-  // g_out (bf16 [B x n_out], its transpose) of the layer above, then layers 3, 2, 1
-  const uint16_t *gb = m->d_Gb, *gbt = m->d_Gbt;
-  int n_out = Kp;
-  for (int l = 2, buf = 0; l >= 0; --l, buf ^= 1) {
-    {
-      EpiArgs e;
-      e.c = m->d_Gz[buf];
-      e.ldc = H;
-      e.z = m->d_Z[l];
-      e.ldz = H;
-      e.a = m->d_Gzb[buf];
-      e.lda = H;
-      e.at = m->d_Gzbt[buf];
-      e.ldat = B;
-      e.ntile = 64;
-      // g_a(l) = g_out * W(l+1): B operand is W(l+1)^T [H x n_out]
-      launch_gemm_tc(3, gb, n_out, m->d_wt[l + 1], n_out, B, H, n_out, e, status, st);
-    }
-    launch_colsum(m->d_Gz[buf], B, H, m->d_g[2 * l + 1], m->d_ws, st);
-    wgrad(m->d_Gzbt[buf], l == 0 ? m->d_Xt : m->d_At[l - 1], H, l == 0 ? F : H, m->d_g[2 * l]);
-    gb = m->d_Gzb[buf];
-    gbt = m->d_Gzbt[buf];
-    n_out = H;
+  launch_train_wgrad(wd, m->stream);
+  for (int t = 0; t < 8; ++t) {
+    ud.rows[t] = m->rows(t);
+    ud.cols[t] = m->cols(t);
+    ud.total += (int64_t)m->rows(t) * m->cols(t);
+    ud.g[t] = m->d_g[t];
+    ud.p[t] = m->d_p[t];
+    ud.m[t] = m->d_m[t];
+    ud.v[t] = m->d_v[t];
   }
-  (void)gbt;
+  ud.adam = adam != nullptr;
+  if (adam) ud.a = *adam;
+  launch_train_update(ud, m->stream);
 }
 
 int check_batch(const ktune_mlp *m, int B) {
@@ -290,21 +286,17 @@ int ktune_mlp_create(ktune_space *s, int K, const int32_t *roles, const float *r
     cudaMemset(m->d_wc, 0, off);
   }
   const size_t B = (size_t)max_batch, H = kMlpHidden;
-  if ((rc = dalloc(&m->d_ws, (size_t)kMlpMaxSplits * kMlpHidden * kMlpMaxF)) ||
+  const size_t n_w = (size_t)H * F + 2 * H * H + (size_t)m->Kp * H;
+  if ((rc = dalloc(&m->d_ws, (size_t)train_splits(max_batch) * n_w)) ||
+      (rc = dalloc(&m->d_part, (size_t)train_part_rows(max_batch) * (3 * H + m->Kp))) ||
       (rc = dalloc(&m->d_range, K)) || (rc = dalloc(&m->d_off, P + 1)) ||
-      (rc = dalloc(&m->d_utab, utab.size())) || (rc = dalloc(&m->d_X, B * F)) ||
-      (rc = dalloc(&m->d_Xt, B * F)) || (rc = dalloc(&m->d_Y, B * m->Kp)) ||
-      (rc = dalloc(&m->d_G, B * m->Kp)) || (rc = dalloc(&m->d_Gb, B * m->Kp)) ||
-      (rc = dalloc(&m->d_Gbt, B * m->Kp)) || (rc = dalloc(&m->d_loss, 1)) ||
-      (rc = dalloc(&m->d_status, 1)))
+      (rc = dalloc(&m->d_utab, utab.size())) || (rc = dalloc(&m->d_Xt, B * F)) ||
+      (rc = dalloc(&m->d_G, B * m->Kp)) || (rc = dalloc(&m->d_Gbt, B * m->Kp)) ||
+      (rc = dalloc(&m->d_loss, 1)) || (rc = dalloc(&m->d_status, 1)))
     return fail(rc);
   for (int l = 0; l < 3; ++l)
-    if ((rc = dalloc(&m->d_Z[l], B * H)) || (rc = dalloc(&m->d_A[l], B * H)) ||
-        (rc = dalloc(&m->d_At[l], B * H)))
-      return fail(rc);
-  for (int b = 0; b < 2; ++b)
-    if ((rc = dalloc(&m->d_Gz[b], B * H)) || (rc = dalloc(&m->d_Gzb[b], B * H)) ||
-        (rc = dalloc(&m->d_Gzbt[b], B * H)))
+    if ((rc = dalloc(&m->d_At[l], B * H)) || (rc = dalloc(&m->d_Gz[l], B * H)) ||
+        (rc = dalloc(&m->d_Gzt[l], B * H)))
       return fail(rc);
   if (cudaMemcpy(m->d_range, ranges, 4 * K, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(m->d_off, m->off.data(), 4 * (P + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -331,15 +323,11 @@ int ktune_mlp_destroy(ktune_mlp *m) {
   }
   cudaFree(m->d_wc);
   for (int l = 0; l < 3; ++l) {
-    cudaFree(m->d_Z[l]);
-    cudaFree(m->d_A[l]);
     cudaFree(m->d_At[l]);
+    cudaFree(m->d_Gz[l]);
+    cudaFree(m->d_Gzt[l]);
   }
-  for (int b = 0; b < 2; ++b) {
-    cudaFree(m->d_Gz[b]);
-    cudaFree(m->d_Gzb[b]);
-    cudaFree(m->d_Gzbt[b]);
-  }
+  cudaFree(m->d_part);
   cudaFree(m->d_ws);
   cudaFree(m->d_range);
   cudaFree(m->d_off);
@@ -347,11 +335,8 @@ int ktune_mlp_destroy(ktune_mlp *m) {
   cudaFree(m->d_data);
   cudaFree(m->d_target);
   cudaFree(m->d_idx);
-  cudaFree(m->d_X);
   cudaFree(m->d_Xt);
-  cudaFree(m->d_Y);
   cudaFree(m->d_G);
-  cudaFree(m->d_Gb);
   cudaFree(m->d_Gbt);
   cudaFree(m->d_loss);
   cudaFree(m->d_status);
@@ -443,7 +428,7 @@ int ktune_mlp_grads(ktune_mlp *m, const int32_t *idx, int B, double *loss, float
   TRY(check_batch(m, B));
   TRY(upload_idx(m, idx, B));
   CK(cudaMemsetAsync(m->d_loss, 0, 8, m->stream));
-  enqueue_fwd_bwd(m, m->d_idx, B);
+  enqueue_step(m, m->d_idx, B, m->d_loss, nullptr);
   CK(cudaGetLastError());
   TRY(finish(m));
   double sse = 0.0;
@@ -475,10 +460,6 @@ int ktune_mlp_train(ktune_mlp *m, const int32_t *idx, int B, int steps, float lr
   }
   const double b1 = 0.9, b2 = 0.999;
   for (int t = 0; t < steps; ++t) {
-    double *lp = losses ? d_losses + t : m->d_loss;
-    std::swap(m->d_loss, lp);
-    enqueue_fwd_bwd(m, m->d_idx + (size_t)t * B, B);
-    std::swap(m->d_loss, lp);
     ++m->adam_t;
     AdamArgs a;
     a.lr = lr;
@@ -489,12 +470,7 @@ int ktune_mlp_train(ktune_mlp *m, const int32_t *idx, int B, int steps, float lr
     a.eps = 1e-8f;
     a.c1 = (float)(1.0 - pow(b1, m->adam_t));
     a.c2 = (float)(1.0 - pow(b2, m->adam_t));
-    for (int p = 0; p < 8; ++p) {
-      const bool w = (p & 1) == 0;
-      const int l = p >> 1;
-      launch_adam(m->d_p[p], m->d_g[p], m->d_m[p], m->d_v[p], m->rows(p), m->cols(p), a,
-                  w ? m->d_wb[l] : nullptr, (w && l > 0) ? m->d_wt[l] : nullptr, m->stream);
-    }
+    enqueue_step(m, m->d_idx + (size_t)t * B, B, losses ? d_losses + t : m->d_loss, &a);
   }
   pack_weights(m);
   const cudaError_t le = cudaGetLastError();
@@ -589,10 +565,7 @@ int ktune_gemm_bf16(const uint16_t *A, int lda, const uint16_t *B, int ldb, floa
   TRY(dalloc(&status, 1));
   cudaStream_t st = (cudaStream_t)stream;
   cudaMemsetAsync(status, 0, 4, st);
-  EpiArgs e;
-  e.c = C;
-  e.ldc = ldc;
-  launch_gemm_tc(0, A, lda, B, ldb, M, N, Kd, e, status, st);
+  launch_gemm_tc(A, lda, B, ldb, M, N, Kd, C, ldc, status, st);
   const cudaError_t le = cudaGetLastError();
   const cudaError_t se = cudaStreamSynchronize(st);
   int h = 0;
