@@ -29,6 +29,7 @@
 
 #include "device_common.cuh"
 #include "internal.h"
+#include "mlp_epi.cuh"
 #include "tc.cuh"
 
 namespace ktune {
@@ -43,13 +44,25 @@ constexpr int kRowThreads = 512;
 constexpr int kActBuf = kRows * kMlpHidden * 2;  // 64 KB
 constexpr int kWBuf = kCols * kMlpHidden * 2;    // 32 KB: 64 x 256 (or K x 256 of the output layer)
 constexpr int kRowSmem = 2 * kActBuf + 2 * kWBuf;
+// tensor-memory columns: the hidden layers' accumulators, the output layer's,
+// a backward layer's, erf(z / sqrt 2) of the hidden layers
+constexpr uint32_t kOutCol = 3 * kCols, kGradCol = 4 * kCols, kErfCol = 5 * kCols;
 
-__device__ __forceinline__ float gelu_f(float z) {
-  return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f));
+// GELU and its derivative from z and erf(z / sqrt 2), which both need.
+__device__ __forceinline__ float gelu_f(float z, float erf) { return 0.5f * z * (1.0f + erf); }
+__device__ __forceinline__ float gelu_grad_f(float z, float erf) {
+  return 0.5f * (1.0f + erf) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
 }
-__device__ __forceinline__ float gelu_grad_f(float z) {
-  return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) +
-         z * expf(-0.5f * z * z) * 0.39894228040143268f;
+
+// 32 lanes x 16 columns into tensor memory; complete after the wait.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]),
+      "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
+      : "memory");
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 // Rows x Kd bf16 (row-major, leading dimension ld) into core matrices with KC = Kd.
@@ -61,13 +74,8 @@ __device__ __forceinline__ void load_rows(uint8_t *dst, const uint16_t *src, int
   }
 }
 
-__device__ __forceinline__ uint4 pack8(const uint16_t *h) {
-  uint4 q;
-  q.x = h[0] | ((uint32_t)h[1] << 16);
-  q.y = h[2] | ((uint32_t)h[3] << 16);
-  q.z = h[4] | ((uint32_t)h[5] << 16);
-  q.w = h[6] | ((uint32_t)h[7] << 16);
-  return q;
+__device__ __forceinline__ void tmem_ld1(uint32_t taddr, float &v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=f"(v) : "r"(taddr));
 }
 
 __device__ __forceinline__ void st_cluster16(uint32_t addr, const uint4 &v) {
@@ -82,7 +90,8 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
   __shared__ uint64_t mbar;
   __shared__ uint32_t tmem_base;
   __shared__ float sh_b[3][kCols], sh_b4[KTUNE_MAX_COUNTERS];
-  __shared__ uint8_t sh_col[kMlpMaxF];             // the parameter of a feature column
+  // a feature column: 4 x parameter (its shift), | 64 for u, 128 for padding; its digit
+  __shared__ uint8_t sh_col[kMlpMaxF], sh_dig[kMlpMaxF];
   __shared__ uint16_t sh_utab[KTUNE_MAX_PARAMS * 16];
   __shared__ int sh_off[KTUNE_MAX_PARAMS + 1];
   uint8_t *const act[2] = {sm, sm + kActBuf};
@@ -113,25 +122,26 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
   for (int c = threadIdx.x; c < F; c += blockDim.x) {
     int j = 0;
     while (j + 1 < td.P && sh_off[j + 1] <= c) ++j;
-    sh_col[c] = (uint8_t)(c >= sh_off[td.P] ? min(c - sh_off[td.P], td.P) : j);
+    const int u = c - sh_off[td.P];
+    sh_col[c] = (uint8_t)(u >= td.P ? 128 : u >= 0 ? 64 | 4 * u : 4 * j);
+    sh_dig[c] = (uint8_t)(c - sh_off[j]);
   }
   __syncthreads();
-  // features: one-hot digits, u per parameter, zeros; four threads per row
+  // features: one-hot digits, u per parameter, zeros; four threads per row, each CTA
+  // of the cluster storing a quarter of the transpose
   for (int G = warp >> 2; G < F / 8; G += 4) {
-    uint16_t v[8];
+    uint32_t v[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const int c = 8 * G + e, j = sh_col[c];
-      uint16_t x = 0;
-      if (live) {
-        if (c >= sh_off[td.P]) x = j < td.P ? sh_utab[j * 16 + nib64(pk, j)] : (uint16_t)0;
-        else x = (int)nib64(pk, j) == c - sh_off[j] ? (uint16_t)0x3F80 : (uint16_t)0;
-      }
-      v[e] = x;
-      // each CTA of the cluster stores a quarter of the transpose
-      if (live && (G & 3) == rank) td.xt[(size_t)c * B + b] = x;
+      const int c = 8 * G + e;
+      const uint32_t m = sh_col[c], dg = (uint32_t)(pk >> (m & 63u)) & 15u;   // 4 x parameter | kind, digit
+      v[e] = !live || (m & 128u) ? 0u : (m & 64u) ? sh_utab[(m & 60u) * 4u + dg] : dg == sh_dig[c] ? 0x3F80u : 0u;
     }
-    *reinterpret_cast<uint4 *>(act[0] + tc::core_off(row, 8 * G, F)) = pack8(v);
+    if (live && (G & 3) == rank)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) td.xt[(size_t)(8 * G + e) * B + b] = (uint16_t)v[e];
+    *reinterpret_cast<uint4 *>(act[0] + tc::core_off(row, 8 * G, F)) =
+        make_uint4(v[0] | v[1] << 16, v[2] | v[3] << 16, v[4] | v[5] << 16, v[6] | v[7] << 16);
   }
   tc::fence_before();
   __syncthreads();
@@ -141,19 +151,21 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
 
   // D[dcol ..) = act * w^T over Kd columns; returns when it is complete and the
   // weights of the layer after the next may be loaded into w's buffer
+  const bool lead = warp == 0 && tc::elect_one();
   auto layer = [&](const uint8_t *a, const uint8_t *w, int Kd, int N, uint32_t dcol) {
     cp_async_wait_group<1>();        // this layer's weights (the next layer's may be in flight)
     tc::fence_async_smem();
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (warp == 0) {                 // the whole warp, so that descriptors live in uniform registers
       tc::fence_async_smem();        // what the other CTAs stored, behind the cluster barrier
       tc::fence_after();
       const uint32_t idesc = tc::idesc_bf16(128, N);
       const uint32_t hi = tc::sdesc_hi((uint32_t)Kd * 16u);
       uint32_t al = tc::sdesc_lo(tc::smem_u32(a), 128), wl = tc::sdesc_lo(tc::smem_u32(w), 128);
       for (int k = 0; k < Kd; k += 16, al += 16, wl += 16)   // 256 bytes per step
-        tc::mma_bf16(tmem + dcol, tc::sdesc_of(al, hi), tc::sdesc_of(wl, hi), idesc, k ? 1u : 0u);
-      tc::mma_commit(&mbar);
+        if (lead) tc::mma_bf16(tmem + dcol, tc::sdesc_of(al, hi), tc::sdesc_of(wl, hi), idesc, k ? 1u : 0u);
+      if (lead) tc::mma_commit(&mbar);
+      __syncwarp();
     }
     bool w_ok = tc::mbar_wait(&mbar, phase, kTrainWait);
     if (!w_ok) w_ok = tc::mbar_wait(&mbar, phase, kTrainWait) && false;   // the MMAs still in flight
@@ -162,8 +174,8 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
     tc::fence_after();
   };
   // 16 bf16 of this thread's row and columns into every CTA's buffer `dst`
-  auto share = [&](uint8_t *dst, const uint16_t (&h)[16]) {
-    const uint4 q0 = pack8(h), q1 = pack8(h + 8);
+  auto share = [&](uint8_t *dst, const uint32_t (&h)[8]) {
+    const uint4 q0 = make_uint4(h[0], h[1], h[2], h[3]), q1 = make_uint4(h[4], h[5], h[6], h[7]);
     const uint32_t at = tc::smem_u32(dst) + tc::core_off(row, n0 + chunk, H);
 #pragma unroll
     for (int r = 0; r < kSplitN; ++r) {
@@ -171,6 +183,13 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
       st_cluster16(p, q0);
       st_cluster16(p + 128u, q1);
     }
+  };
+  // the same into the transpose [256][B] of a layer
+  auto store_t = [&](uint16_t *t, const uint32_t (&h)[8]) {
+    if (live)
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        t[(size_t)(n0 + chunk + i) * B + b] = (uint16_t)(i & 1 ? h[i >> 1] >> 16 : h[i >> 1]);
   };
   auto barrier = [&]() {
     asm volatile("fence.proxy.async;" ::: "memory");
@@ -188,86 +207,92 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
     else if (l == 1) load_rows(wb[1], td.w[3], H, Kp, H);
     else load_rows(wb[0], td.wt[3] + (size_t)n0 * Kp, Kp, kCols, Kp);
     cp_async_commit();
-    float v[16];
-    uint16_t h[16];
+    float v[16], erf[16];
+    uint32_t h[8];
     tc::tmem_ld16(tmem + lanes + (uint32_t)(l * kCols + chunk), v);
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      h[i] = tc::f2bf(gelu_f(__fadd_rn(v[i], sh_b[l][chunk + i])));
-      if (live) td.at[l][(size_t)(n0 + chunk + i) * B + b] = h[i];
+      const float z = __fadd_rn(v[i], sh_b[l][chunk + i]);
+      erf[i] = erff(z * 0.70710678118654752f);
+      v[i] = gelu_f(z, erf[i]);
     }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) h[i] = bf2(v[2 * i], v[2 * i + 1]);
     share(act[(l + 1) & 1], h);
+    store_t(td.at[l], h);
+    tmem_st16(tmem + lanes + kErfCol + (uint32_t)(l * kCols + chunk), erf);
     barrier();
   }
-  // ---- output layer, loss and its gradient (every CTA of the cluster, its own copy) ----
+  // ---- output layer (every CTA all of it), loss and its gradient (a quarter of the
+  // columns per CTA, a sixteenth per thread, shared like the activations) --------------
+  double e = 0.0;
   {
-    float t[16];
-    const bool mine = chunk < Kp;
+    const int nc = Kp >> 4, c0 = rank * (Kp >> 2) + (warp >> 2) * nc;
+    float t[4], v[4];
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
-      t[i] = live && chunk + i < K ? td.target[(size_t)src * K + chunk + i] : 0.0f;
-    layer(act[1], wb[1], H, Kp, 3u * kCols);
+    for (int i = 0; i < 4; ++i)
+      t[i] = i < nc && live && c0 + i < K ? td.target[(size_t)src * K + c0 + i] : 0.0f;
+    layer(act[1], wb[1], H, Kp, kOutCol);
     load_rows(wb[1], td.wt[2] + (size_t)n0 * H, H, kCols, H);
     cp_async_commit();
-    double e = 0.0;
-    if (mine) {
-      float v[16], g[16];
-      uint16_t h[16];
-      tc::tmem_ld16(tmem + lanes + (uint32_t)(3 * kCols + chunk), v);
-      const float bk = (float)B * (float)K;      // below 2^24: exact
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        g[i] = 0.0f;
-        if (live && chunk + i < K) {
-          const float d = __fsub_rn(__fadd_rn(v[i], sh_b4[chunk + i]), t[i]);
-          if ((i >> 2) == rank) e += (double)d * (double)d;
-          // 2 d / (B K), one rounding (a float64 quotient rounded to float32 is the same number)
-          g[i] = __fdiv_rn(2.0f * d, bk);
-        }
-        h[i] = tc::f2bf(g[i]);
-        if (live && (i >> 2) == rank) td.gbt[(size_t)(chunk + i) * B + b] = h[i];
+    for (int i = 0; i < 4; ++i) tmem_ld1(tmem + lanes + kOutCol + (uint32_t)min(c0 + i, Kp - 1), v[i]);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3])::"memory");
+    const float bk = (float)B * (float)K;      // below 2^24: exact
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (i >= nc) break;
+      float g = 0.0f;
+      if (live && c0 + i < K) {
+        const float d = __fsub_rn(__fadd_rn(v[i], sh_b4[c0 + i]), t[i]);
+        e += (double)d * (double)d;
+        // 2 d / (B K), one rounding (a float64 quotient rounded to float32 is the same number)
+        g = __fdiv_rn(2.0f * d, bk);
       }
-      if (live)
+      const uint16_t h = (uint16_t)bf2(g, 0.0f);
+      const uint32_t at = tc::smem_u32(act[0]) + tc::core_off(row, c0 + i, Kp);
 #pragma unroll
-        for (int i = 0; i < 16; i += 4)
-          if ((i >> 2) == rank)
-            *reinterpret_cast<float4 *>(td.g + (size_t)b * Kp + chunk + i) =
-                make_float4(g[i], g[i + 1], g[i + 2], g[i + 3]);
-      *reinterpret_cast<uint4 *>(act[0] + tc::core_off(row, chunk, Kp)) = pack8(h);
-      *reinterpret_cast<uint4 *>(act[0] + tc::core_off(row, chunk + 8, Kp)) = pack8(h + 8);
+      for (int r = 0; r < kSplitN; ++r)
+        asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(tc::map_rank(at, (uint32_t)r)), "h"(h) : "memory");
+      if (live) {
+        td.gbt[(size_t)(c0 + i) * B + b] = h;
+        td.g[(size_t)b * Kp + c0 + i] = g;
+      }
     }
-    for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-    if (lane == 0 && e != 0.0) atomicAdd(td.loss, e);
-    barrier();               // every CTA's output layer has read its activations
+    barrier();
   }
   // ---- backward: g_z(l) = (g(l + 1) W(l + 1)) GELU'(z(l)), l = 2, 1, 0 -------------------
 #pragma unroll 1
   for (int l = 2; l >= 0; --l) {
     const int s = l & 1;                       // l = 2: act[0], wb[0]; 1: act[1], wb[1]; 0: act[0], wb[0]
-    const uint32_t dcol = 256u + (uint32_t)(l * kCols);
-    layer(act[s], wb[s], l == 2 ? Kp : H, kCols, dcol);
+    layer(act[s], wb[s], l == 2 ? Kp : H, kCols, kGradCol);
     if (l == 2) load_rows(wb[0], td.wt[1] + (size_t)n0 * H, H, kCols, H);
     cp_async_commit();
-    float v[16], z[16];
-    uint16_t h[16];
-    tc::tmem_ld16(tmem + lanes + (uint32_t)(l * kCols + chunk), z);
-    tc::tmem_ld16(tmem + lanes + dcol + (uint32_t)chunk, v);
+    float v[16];
+    uint32_t h[8];
+    {
+      float z[16], erf[16];
+      tc::tmem_ld16(tmem + lanes + (uint32_t)(l * kCols + chunk), z);
+      tc::tmem_ld16(tmem + lanes + kErfCol + (uint32_t)(l * kCols + chunk), erf);
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      v[i] = __fmul_rn(v[i], gelu_grad_f(__fadd_rn(z[i], sh_b[l][chunk + i])));
-      h[i] = tc::f2bf(v[i]);
-      if (live) td.gzt[l][(size_t)(n0 + chunk + i) * B + b] = h[i];
+      for (int i = 0; i < 16; ++i) z[i] = gelu_grad_f(__fadd_rn(z[i], sh_b[l][chunk + i]), erf[i]);
+      tc::tmem_ld16(tmem + lanes + kGradCol + (uint32_t)chunk, v);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] = __fmul_rn(v[i], z[i]);
     }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) h[i] = bf2(v[2 * i], v[2 * i + 1]);
+    if (l > 0) share(act[s ^ 1], h);
+    store_t(td.gzt[l], h);
     if (live)
 #pragma unroll
       for (int i = 0; i < 16; i += 4)
         *reinterpret_cast<float4 *>(td.gz[l] + (size_t)b * H + n0 + chunk + i) =
             make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-    if (l > 0) {
-      share(act[s ^ 1], h);
-      barrier();
-    }
+    if (l > 0) barrier();
   }
+  for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+  if (lane == 0 && e != 0.0) atomicAdd(td.loss, e);
   cp_async_wait_all();
   if (!ok && threadIdx.x == 0) atomicExch(td.status, KTUNE_ETIMEOUT);
   tc::fence_before();
