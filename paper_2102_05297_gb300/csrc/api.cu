@@ -173,10 +173,10 @@ int build_groups(ktune_space *s, const int32_t *code, int n) {
   return KTUNE_OK;
 }
 
-// Constrained-index table (see kCiMaxBits): built when the constrained
-// parameters' value combinations number at most kCiMaxBits and there is at
-// least one constraint; every combination is checked against every group's
-// table.
+// Shape of the constrained-index table (see kCiMaxBits): there is one when the
+// constrained parameters' value combinations number at most kCiMaxBits and there
+// is at least one constraint.  Its bits are computed on the device
+// (k_ci_table: up to 131,072 combinations, 0.9 ms on one host thread).
 void build_ci(ktune_space *s) {
   if (s->groups.empty()) return;
   uint32_t used = 0;
@@ -192,17 +192,7 @@ void build_ci(ktune_space *s) {
         return;
       }
     }
-  s->ci_table.assign((size_t)((prod + 31) / 32), 0u);
-  for (int64_t c = 0; c < prod; ++c) {
-    uint64_t p = 0;   // packed digits of a configuration with this constrained combination
-    int64_t rem = c;
-    for (int j = s->sa.P - 1; j >= 0; --j)
-      if ((used >> j) & 1u) {
-        p |= (uint64_t)(rem % s->sa.radix[j]) << (4 * j);
-        rem /= s->sa.radix[j];
-      }
-    if (ktune::host_valid(s, p)) s->ci_table[(size_t)(c >> 5)] |= 1u << (c & 31);
-  }
+  s->ci_combos = prod;
 }
 
 // Window tables of the one-word layout (see WinDev): groups in program order
@@ -486,14 +476,6 @@ int ktune_space_create(const ktune_space_desc *d, int flags, void *stream, ktune
   if ((rc = dalloc(&s->d_groups, s->groups.size()))) return cleanup(rc);
   if ((rc = dalloc(&s->d_table, s->table.size()))) return cleanup(rc);
   if ((rc = dalloc(&s->d_win_table, std::max<size_t>(1, s->win_table.size())))) return cleanup(rc);
-  if (!s->ci_table.empty()) {
-    if ((rc = dalloc(&s->d_ci_table, s->ci_table.size()))) return cleanup(rc);
-    if (cudaMemcpyAsync(s->d_ci_table, s->ci_table.data(), s->ci_table.size() * 4,
-                        cudaMemcpyHostToDevice, (cudaStream_t)stream) != cudaSuccess) {
-      set_error("descriptor upload failed");
-      return cleanup(KTUNE_ECUDA);
-    }
-  }
   if (!s->win_table.empty() &&
       cudaMemcpyAsync(s->d_win_table, s->win_table.data(), s->win_table.size() * 4,
                       cudaMemcpyHostToDevice, (cudaStream_t)stream) != cudaSuccess) {
@@ -509,19 +491,48 @@ int ktune_space_create(const ktune_space_desc *d, int flags, void *stream, ktune
       return cleanup(KTUNE_ECUDA);
     }
   }
+  CiArgs ci{};
+  if (s->ci_combos) {
+    ci.words = (int)((s->ci_combos + 31) / 32);
+    for (int j = 0; j < s->sa.P; ++j) ci.stride[j] = s->ci_stride[j];
+    if ((rc = dalloc(&s->d_ci_table, ci.words))) return cleanup(rc);
+    launch_ci_table(s->sa, s->d_groups, s->d_table, ci, s->ci_combos, s->d_ci_table, cs);
+    ci.table = s->d_ci_table;
+  }
   s->n_tiles = (s->sa.n_raw + kEnumTileRaw - 1) / kEnumTileRaw;
+  // scratch of the enumeration: the tiles' counts and, for the writing pass of a
+  // materialised space, the runs' valid bits (up to 128 MB; larger raw spaces are
+  // checked again there)
   int32_t *d_count = nullptr;
-  if ((rc = dalloc(&d_count, s->n_tiles))) return cleanup(rc);
-  if ((rc = dalloc(&s->d_tile_offset, s->n_tiles + 1))) {
+  uint16_t *d_masks = nullptr;
+  auto drop = [&]() {
     cudaFree(d_count);
+    cudaFree(d_masks);
+  };
+  if ((rc = dalloc(&d_count, s->n_tiles)) || (rc = dalloc(&s->d_tile_offset, s->n_tiles + 1)) ||
+      (flags == KTUNE_MATERIALISE && s->sa.n_raw <= (int64_t)1 << 30 &&
+       (rc = dalloc(&d_masks, s->n_tiles * kEnumThreads)))) {
+    drop();
     return cleanup(rc);
   }
-  launch_enum_count(s->sa, s->d_groups, s->d_table, s->n_tiles, d_count, cs);
+  launch_enum_count(s->sa, s->d_groups, s->d_table, ci, s->n_tiles, d_count, d_masks, cs);
   launch_scan_tiles(d_count, s->n_tiles, s->d_tile_offset, cs);
   cudaError_t e = cudaMemcpyAsync(&s->n_valid, s->d_tile_offset + s->n_tiles, sizeof(int64_t),
                                   cudaMemcpyDeviceToHost, cs);
   if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
-  cudaFree(d_count);
+  if (e == cudaSuccess && flags == KTUNE_MATERIALISE) {
+    WordArgs wa{};
+    for (int j = 0; j < s->sa.P; ++j) wa.pos[j] = s->pos[j];
+    if ((rc = dalloc(&s->d_packed, s->n_valid)) || (s->narrow && (rc = dalloc(&s->d_narrow, s->n_valid)))) {
+      drop();
+      return cleanup(rc);
+    }
+    launch_enum_write(s->sa, s->d_groups, s->d_table, d_masks, s->n_tiles, s->d_tile_offset, s->d_packed,
+                      wa, s->d_narrow, cs);
+    e = cudaStreamSynchronize(cs);
+    if (e == cudaSuccess) e = cudaGetLastError();
+  }
+  drop();
   if (e != cudaSuccess) {
     set_error(std::string("enumeration: ") + cudaGetErrorString(e));
     return cleanup(KTUNE_ECUDA);
@@ -545,23 +556,6 @@ int ktune_space_create(const ktune_space_desc *d, int flags, void *stream, ktune
         set_error("tile list upload failed");
         return cleanup(KTUNE_ECUDA);
       }
-    }
-  }
-  if (flags == KTUNE_MATERIALISE) {
-    if ((rc = dalloc(&s->d_packed, s->n_valid))) return cleanup(rc);
-    launch_enum_write(s->sa, s->d_groups, s->d_table, s->n_tiles, s->d_tile_offset, s->d_packed,
-                      cs);
-    if (s->narrow) {
-      if ((rc = dalloc(&s->d_narrow, s->n_valid))) return cleanup(rc);
-      PrepArgs lay{};
-      for (int j = 0; j < s->sa.P; ++j) lay.pos[j] = s->pos[j];
-      launch_narrow_pack(s->d_packed, s->n_valid, lay, s->d_narrow, cs);
-    }
-    e = cudaStreamSynchronize(cs);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      set_error(std::string("enumeration: ") + cudaGetErrorString(e));
-      return cleanup(KTUNE_ECUDA);
     }
   }
   *out = s;
@@ -597,10 +591,38 @@ int ktune_space_decode(const ktune_space *s, int64_t raw, int64_t *values_out) {
   return KTUNE_OK;
 }
 
+// Read-back of a range of TS: from kReadOnDevice configurations on, converted by
+// a kernel into a temporary device buffer and copied straight to the caller
+// (2.26M raw indices: 8.7 ms on one host thread, see ktune_space_valid_raw);
+// below, the packed digits are copied and converted here (a few tens of
+// microseconds, no allocation).
+extern "C++" {
+namespace {
+constexpr int64_t kReadOnDevice = 8192;
+template <typename F>
+int read_device(int64_t bytes, void *out, F convert, int64_t out_bytes = -1) {
+  uint8_t *tmp = nullptr;
+  TRY(dalloc(&tmp, (size_t)bytes));
+  convert(tmp);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = cudaMemcpy(out, tmp, out_bytes < 0 ? bytes : out_bytes, cudaMemcpyDeviceToHost);
+  cudaFree(tmp);
+  if (e != cudaSuccess) FAIL(KTUNE_ECUDA, std::string("read-back: ") + cudaGetErrorString(e));
+  return KTUNE_OK;
+}
+}  // namespace
+}  // extern "C++"
+
 int ktune_space_valid_raw(const ktune_space *s, int64_t first, int64_t count, int64_t *out_raw) {
   if (!s || (!out_raw && count)) FAIL(KTUNE_EINVAL, "null argument");
   if (!s->d_packed) FAIL(KTUNE_ESTATE, "space is not materialised");
   if (first < 0 || count < 0 || first + count > s->n_valid) FAIL(KTUNE_EINVAL, "range out of TS");
+  if (count >= kReadOnDevice) {
+    return read_device(count * 8, out_raw, [&](void *tmp) {
+      launch_raw_of(s->d_packed + first, count, s->sa, static_cast<int64_t *>(tmp), nullptr);
+    });
+  }
   std::vector<uint64_t> p((size_t)count);
   if (count) CK(cudaMemcpy(p.data(), s->d_packed + first, count * 8, cudaMemcpyDeviceToHost));
   for (int64_t i = 0; i < count; ++i) {
@@ -615,6 +637,11 @@ int ktune_space_valid_digits(const ktune_space *s, int64_t first, int64_t count,
   if (!s || (!out && count)) FAIL(KTUNE_EINVAL, "null argument");
   if (!s->d_packed) FAIL(KTUNE_ESTATE, "space is not materialised");
   if (first < 0 || count < 0 || first + count > s->n_valid) FAIL(KTUNE_EINVAL, "range out of TS");
+  if (count >= kReadOnDevice) {
+    return read_device((count * s->sa.P + 3) / 4 * 4, out, [&](void *tmp) {
+      launch_digits_of(s->d_packed + first, count, s->sa.P, static_cast<uint32_t *>(tmp), nullptr);
+    }, count * s->sa.P);
+  }
   std::vector<uint64_t> p((size_t)count);
   if (count) CK(cudaMemcpy(p.data(), s->d_packed + first, count * 8, cudaMemcpyDeviceToHost));
   const int P = s->sa.P;
@@ -1007,7 +1034,7 @@ int ktune_search_create(ktune_space *s, ktune_model *m, const ktune_search_opts 
     sd.width[j] = s->width[j];
   }
   sd.ci_table = s->d_ci_table;
-  sd.ci_words = (int)s->ci_table.size();
+  sd.ci_words = (int)((s->ci_combos + 31) / 32);
   for (int j = 0; j < KTUNE_MAX_PARAMS; ++j) sd.ci_stride[j] = s->ci_stride[j];
   sd.win_table = s->d_win_table;
   sd.n_win = (int)s->win.size();

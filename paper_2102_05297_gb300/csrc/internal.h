@@ -258,13 +258,28 @@ void launch_bweights(const SearchDev *srch, const int *sub_search, int64_t n_sub
 void launch_bselect(const SearchDev *srch, const StepDev *steps, int S, cudaStream_t st);
 
 // ---- enumeration (k_space.cu) ----
-void launch_enum_count(const SpaceArgs &sa, const GroupDev *groups, const uint32_t *table,
-                       int64_t n_tiles, int32_t *tile_count, cudaStream_t st);
+// The constrained-index table as the enumeration reads it (table null: none).
+struct CiArgs {
+  const uint32_t *table;
+  int words;
+  uint32_t stride[KTUNE_MAX_PARAMS];
+};
+struct WordArgs {
+  uint8_t pos[KTUNE_MAX_PARAMS];        // the one-word form's bit positions
+};
+void launch_ci_table(const SpaceArgs &sa, const GroupDev *groups, const uint32_t *table, const CiArgs &ci,
+                     int64_t combos, uint32_t *out, cudaStream_t st);
+// masks: 16 valid bits per run of 16 raw indices (null: not kept)
+void launch_enum_count(const SpaceArgs &sa, const GroupDev *groups, const uint32_t *table, const CiArgs &ci,
+                       int64_t n_tiles, int32_t *tile_count, uint16_t *masks, cudaStream_t st);
 void launch_scan_tiles(const int32_t *tile_count, int64_t n_tiles, int64_t *tile_offset,
                        cudaStream_t st);
 void launch_enum_write(const SpaceArgs &sa, const GroupDev *groups, const uint32_t *table,
-                       int64_t n_tiles, const int64_t *tile_offset, uint64_t *packed,
-                       cudaStream_t st);
+                       const uint16_t *masks, int64_t n_tiles, const int64_t *tile_offset, uint64_t *packed,
+                       const WordArgs &wa, uint32_t *narrow, cudaStream_t st);
+void launch_raw_of(const uint64_t *packed, int64_t n, const SpaceArgs &sa, int64_t *raw, cudaStream_t st);
+// out: n * P bytes, rounded up to whole words
+void launch_digits_of(const uint64_t *packed, int64_t n, int P, uint32_t *out, cudaStream_t st);
 
 // ---- search step (k_step.cu) ----
 // (the allocation-free scoring path: each returns the launch's own status)
@@ -277,8 +292,6 @@ cudaError_t score_mat_device_setup();
 cudaError_t launch_score_mat(const uint64_t *packed, const uint32_t *evaluated, int64_t N,
                              const uint8_t *pack, const int *n_active, int D, float *s,
                              float2 *minmax, int grid, cudaStream_t st);
-void launch_narrow_pack(const uint64_t *packed, int64_t n, const PrepArgs &layout,
-                        uint32_t *narrow, cudaStream_t st);
 void launch_predict_full(const uint64_t *packed, int64_t count, const uint8_t *nodes,
                          const float *leaves, int K, int D, float *out, cudaStream_t st);
 void launch_mark(uint32_t *evaluated, int64_t ordinal, cudaStream_t st);
@@ -464,7 +477,7 @@ struct ktune_space {
   std::vector<uint8_t> generic;      // groups no window covers
   uint32_t *d_win_table = nullptr;
   // constrained-index table (narrow spaces whose constrained combinations fit)
-  std::vector<uint32_t> ci_table;
+  int64_t ci_combos = 0;             // combinations (0: no table)
   uint32_t ci_stride[KTUNE_MAX_PARAMS] = {0};
   uint32_t *d_ci_table = nullptr;
 };

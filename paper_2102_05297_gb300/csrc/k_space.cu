@@ -4,9 +4,17 @@
 // array TS), with block-scan compaction into ascending raw order.
 //
 // Work split: one CTA per tile of kEnumTileRaw consecutive raw indices, each
-// thread a run of 16 consecutive indices (decoded once by division, then
-// advanced by an odometer increment on the packed nibbles).  Constraints are
-// evaluated through per-group bit tables built on the host from the bytecode.
+// thread a run of 16 consecutive indices (decoded once by 32-bit divisions where
+// the raw size allows, then advanced by an odometer increment on the packed
+// nibbles).  Constraints are evaluated through the constrained-index table (one
+// bit per combination of the constrained parameters, one shared-memory load per
+// raw index; the odometer carries the index along) or, where that table would
+// be too large, through per-group bit tables.  The counting pass keeps each
+// run's 16 valid bits (raw size / 8 bytes), so that the writing pass decodes
+// only runs that hold a valid configuration.  What bounds the counting pass is
+// the instructions per raw index (odometer, bit).  41.3M raw, 2.26M valid
+// configurations: 290 + 306 + 12 us with a table load and a digit sum per
+// constraint group in both passes and a third pass for the one-word form.
 #include "internal.h"
 
 namespace ktune {
@@ -61,14 +69,24 @@ __device__ __forceinline__ void load_groups(SmemGroups &sg, const GroupDev *grou
   __syncthreads();
 }
 
-// Per thread: bitmask of valid indices in its run and the run's first digits.
+__device__ __forceinline__ uint64_t decode_run(const SpaceArgs &sa, int64_t raw) {
+  if (sa.n_raw > 0xffffffffll) return decode_packed(sa, raw);
+  uint64_t packed = 0;
+  uint32_t r = (uint32_t)raw;
+  for (int j = sa.P - 1; j >= 0; --j) {
+    const uint32_t q = r / (uint32_t)sa.radix[j];
+    packed |= (uint64_t)(r - q * (uint32_t)sa.radix[j]) << (4 * j);
+    r = q;
+  }
+  return packed;
+}
+
+// Bitmask of the valid indices of the run at r0.
 __device__ __forceinline__ uint32_t run_mask(const SpaceArgs &sa, const SmemGroups &sg,
-                                             const uint32_t *table, int64_t r0,
-                                             uint64_t *first) {
+                                             const uint32_t *table, int64_t r0) {
   uint32_t mask = 0;
   if (r0 >= sa.n_raw) return 0;
-  uint64_t p = decode_packed(sa, r0);
-  *first = p;
+  uint64_t p = decode_run(sa, r0);
   const int64_t left = sa.n_raw - r0;
   const int n = left < kRunLen ? (int)left : kRunLen;
   for (int i = 0; i < n; ++i) {
@@ -78,16 +96,51 @@ __device__ __forceinline__ uint32_t run_mask(const SpaceArgs &sa, const SmemGrou
   return mask;
 }
 
-__global__ void __launch_bounds__(kEnumThreads) k_enum_count(SpaceArgs sa, const GroupDev *groups,
-                                                             const uint32_t *table, int64_t n_tiles,
-                                                             int32_t *tile_count) {
+// The same through the constrained-index table.
+__device__ __forceinline__ uint32_t run_mask_ci(const SpaceArgs &sa, const CiArgs &ci, const uint32_t *tab,
+                                                int64_t r0) {
+  uint32_t mask = 0;
+  if (r0 >= sa.n_raw) return 0;
+  uint64_t p = decode_run(sa, r0);
+  uint32_t c = 0;
+  for (int j = 0; j < sa.P; ++j) c += nib(p, j) * ci.stride[j];
+  const int64_t left = sa.n_raw - r0;
+  const int n = left < kRunLen ? (int)left : kRunLen;
+  for (int i = 0; i < n; ++i) {
+    mask |= ((tab[c >> 5] >> (c & 31u)) & 1u) << i;
+    for (int j = sa.P - 1; j >= 0; --j) {      // one step of the odometer
+      const uint32_t d = nib(p, j) + 1;
+      if (d < (uint32_t)sa.radix[j]) {
+        p += 1ull << (4 * j);
+        c += ci.stride[j];
+        break;
+      }
+      p &= ~(15ull << (4 * j));
+      c -= (d - 1) * ci.stride[j];
+    }
+  }
+  return mask;
+}
+
+template <bool CI>
+__global__ void __launch_bounds__(kEnumThreads)
+    k_enum_count(const __grid_constant__ SpaceArgs sa, const GroupDev *groups, const uint32_t *table,
+                 const __grid_constant__ CiArgs ci, int64_t n_tiles, int32_t *tile_count,
+                 uint16_t *masks) {
+  extern __shared__ uint32_t tab[];
   __shared__ SmemGroups sg;
   __shared__ int warp_sum[kEnumThreads / 32];
-  load_groups(sg, groups, sa.n_groups);
+  if (CI) {
+    for (int i = threadIdx.x; i < ci.words; i += blockDim.x) tab[i] = ci.table[i];
+    __syncthreads();
+  } else {
+    load_groups(sg, groups, sa.n_groups);
+  }
   for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    int64_t r0 = t * kEnumTileRaw + (int64_t)threadIdx.x * kRunLen;
-    uint64_t first;
-    int c = __popc(run_mask(sa, sg, table, r0, &first));
+    const int64_t r0 = t * kEnumTileRaw + (int64_t)threadIdx.x * kRunLen;
+    const uint32_t m = CI ? run_mask_ci(sa, ci, tab, r0) : run_mask(sa, sg, table, r0);
+    if (masks) masks[t * kEnumThreads + threadIdx.x] = (uint16_t)m;
+    int c = __popc(m);
     for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = c;
     __syncthreads();
@@ -100,18 +153,21 @@ __global__ void __launch_bounds__(kEnumThreads) k_enum_count(SpaceArgs sa, const
   }
 }
 
-__global__ void __launch_bounds__(kEnumThreads) k_enum_write(SpaceArgs sa, const GroupDev *groups,
-                                                             const uint32_t *table, int64_t n_tiles,
-                                                             const int64_t *tile_offset,
-                                                             uint64_t *packed_out) {
+// The valid configurations at their ordinals: packed digits and, for spaces
+// with a one-word form, that form.
+__global__ void __launch_bounds__(kEnumThreads)
+    k_enum_write(const __grid_constant__ SpaceArgs sa, const GroupDev *groups, const uint32_t *table,
+                 const uint16_t *masks, int64_t n_tiles, const int64_t *tile_offset,
+                 uint64_t *packed_out, const __grid_constant__ WordArgs wa, uint32_t *narrow_out) {
   __shared__ SmemGroups sg;
   __shared__ int warp_sum[kEnumThreads / 32];
-  load_groups(sg, groups, sa.n_groups);
+  if (!masks) load_groups(sg, groups, sa.n_groups);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    int64_t r0 = t * kEnumTileRaw + (int64_t)threadIdx.x * kRunLen;
-    uint64_t p = 0;
-    uint32_t mask = run_mask(sa, sg, table, r0, &p);
+    const int64_t lo = tile_offset[t];
+    if (lo == tile_offset[t + 1]) continue;    // the same for the whole block
+    const int64_t r0 = t * kEnumTileRaw + (int64_t)threadIdx.x * kRunLen;
+    uint32_t mask = masks ? masks[t * kEnumThreads + threadIdx.x] : run_mask(sa, sg, table, r0);
     int c = __popc(mask);
     // exclusive scan of c over the block (thread order = raw order)
     int incl = c;
@@ -123,14 +179,76 @@ __global__ void __launch_bounds__(kEnumThreads) k_enum_write(SpaceArgs sa, const
     __syncthreads();
     int base = 0;
     for (int w = 0; w < warp; ++w) base += warp_sum[w];
-    int64_t pos = tile_offset[t] + base + incl - c;
-    for (int i = 0; mask; ++i) {
-      if (mask & 1u) packed_out[pos++] = p;
-      mask >>= 1;
-      p = odometer_next(sa, p);
+    int64_t pos = lo + base + incl - c;
+    if (mask) {
+      uint64_t p = decode_run(sa, r0);
+      for (; mask; mask >>= 1) {
+        if (mask & 1u) {
+          packed_out[pos] = p;
+          if (narrow_out) {
+            uint32_t w = 0;
+            for (int j = 0; j < sa.P; ++j) w |= nib(p, j) << wa.pos[j];
+            narrow_out[pos] = w;
+          }
+          ++pos;
+        }
+        p = odometer_next(sa, p);
+      }
     }
     __syncthreads();
   }
+}
+
+// Constrained-index table: bit c says whether the combination c of the
+// constrained parameters satisfies every group.
+__global__ void k_ci_table(const __grid_constant__ SpaceArgs sa, const GroupDev *groups, const uint32_t *table,
+                           const __grid_constant__ CiArgs ci, int64_t combos, uint32_t *out) {
+  __shared__ SmemGroups sg;
+  load_groups(sg, groups, sa.n_groups);
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  bool ok = false;
+  if (c < combos) {
+    uint64_t p = 0;
+    uint32_t rem = (uint32_t)c;
+    for (int j = sa.P - 1; j >= 0; --j)
+      if (ci.stride[j]) {
+        const uint32_t q = rem / (uint32_t)sa.radix[j];
+        p |= (uint64_t)(rem - q * (uint32_t)sa.radix[j]) << (4 * j);
+        rem = q;
+      }
+    ok = valid_packed(p, sg.g, sa.n_groups, table);
+  }
+  const uint32_t bits = __ballot_sync(0xffffffffu, ok);
+  if ((threadIdx.x & 31) == 0 && c < combos) out[c >> 5] = bits;
+}
+
+// Raw indices of packed configurations.
+__global__ void k_raw_of(const uint64_t *__restrict__ packed, int64_t n, const __grid_constant__ SpaceArgs sa,
+                         int64_t *__restrict__ raw) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const uint64_t p = packed[i];
+  int64_t r = 0;
+  for (int j = 0; j < sa.P; ++j) r += (int64_t)nib(p, j) * sa.stride[j];
+  raw[i] = r;
+}
+
+// Digits as bytes [n][P], four bytes per thread.
+__global__ void k_digits_of(const uint64_t *__restrict__ packed, int64_t n, int P, uint32_t *__restrict__ out) {
+  const int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t bytes = n * P;
+  if (w * 4 >= bytes) return;
+  int64_t i = w * 4 / P;
+  int j = (int)(w * 4 - i * P);
+  uint32_t v = 0;
+  for (int e = 0; e < 4 && w * 4 + e < bytes; ++e) {
+    v |= nib(packed[i], j) << (8 * e);
+    if (++j == P) {
+      j = 0;
+      ++i;
+    }
+  }
+  out[w] = v;
 }
 
 // Exclusive prefix sum of the tile counts (one CTA); tile_offset[n_tiles] = total.
@@ -170,9 +288,19 @@ int enum_grid(int64_t n_tiles) {
 
 }  // namespace
 
-void launch_enum_count(const SpaceArgs &sa, const GroupDev *groups, const uint32_t *table,
-                       int64_t n_tiles, int32_t *tile_count, cudaStream_t st) {
-  k_enum_count<<<enum_grid(n_tiles), kEnumThreads, 0, st>>>(sa, groups, table, n_tiles, tile_count);
+void launch_ci_table(const SpaceArgs &sa, const GroupDev *groups, const uint32_t *table, const CiArgs &ci,
+                     int64_t combos, uint32_t *out, cudaStream_t st) {
+  k_ci_table<<<(unsigned)((combos + 255) / 256), 256, 0, st>>>(sa, groups, table, ci, combos, out);
+}
+
+void launch_enum_count(const SpaceArgs &sa, const GroupDev *groups, const uint32_t *table, const CiArgs &ci,
+                       int64_t n_tiles, int32_t *tile_count, uint16_t *masks, cudaStream_t st) {
+  if (ci.table)
+    k_enum_count<true><<<enum_grid(n_tiles), kEnumThreads, ci.words * 4, st>>>(sa, groups, table, ci, n_tiles,
+                                                                               tile_count, masks);
+  else
+    k_enum_count<false><<<enum_grid(n_tiles), kEnumThreads, 0, st>>>(sa, groups, table, ci, n_tiles,
+                                                                     tile_count, masks);
 }
 
 void launch_scan_tiles(const int32_t *tile_count, int64_t n_tiles, int64_t *tile_offset,
@@ -181,10 +309,18 @@ void launch_scan_tiles(const int32_t *tile_count, int64_t n_tiles, int64_t *tile
 }
 
 void launch_enum_write(const SpaceArgs &sa, const GroupDev *groups, const uint32_t *table,
-                       int64_t n_tiles, const int64_t *tile_offset, uint64_t *packed,
-                       cudaStream_t st) {
-  k_enum_write<<<enum_grid(n_tiles), kEnumThreads, 0, st>>>(sa, groups, table, n_tiles,
-                                                            tile_offset, packed);
+                       const uint16_t *masks, int64_t n_tiles, const int64_t *tile_offset, uint64_t *packed,
+                       const WordArgs &wa, uint32_t *narrow, cudaStream_t st) {
+  k_enum_write<<<enum_grid(n_tiles), kEnumThreads, 0, st>>>(sa, groups, table, masks, n_tiles, tile_offset,
+                                                            packed, wa, narrow);
+}
+
+void launch_raw_of(const uint64_t *packed, int64_t n, const SpaceArgs &sa, int64_t *raw, cudaStream_t st) {
+  k_raw_of<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(packed, n, sa, raw);
+}
+
+void launch_digits_of(const uint64_t *packed, int64_t n, int P, uint32_t *out, cudaStream_t st) {
+  k_digits_of<<<(unsigned)((n * P + 1023) / 1024), 256, 0, st>>>(packed, n, P, out);
 }
 
 }  // namespace ktune

@@ -6,7 +6,6 @@
 //   k_score_mat    every configuration: walk the active trees (two-word
 //                  digits), sum the terms (Eq. score), CTA min/max
 //   k_predict_full all K counters of a range of TS (Section 3.3.2)
-//   k_narrow_pack  TS in the one-word digit layout
 #include <float.h>
 
 #include "device_common.cuh"
@@ -190,16 +189,6 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
   }
 }
 
-__global__ void k_narrow_pack(const uint64_t *__restrict__ packed, int64_t n, PrepArgs lay,
-                              uint32_t *__restrict__ out) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint64_t p = packed[i];
-  uint32_t w = 0;
-  for (int j = 0; j < KTUNE_MAX_PARAMS; ++j) w |= nib64(p, j) << lay.pos[j];
-  out[i] = w;
-}
-
 __global__ void k_predict_full(const uint64_t *__restrict__ packed, int64_t count,
                                const uint8_t *__restrict__ nodes, const float *__restrict__ leaves,
                                int K, int D, float *__restrict__ out) {
@@ -258,12 +247,6 @@ cudaError_t launch_score_mat(const uint64_t *packed, const uint32_t *evaluated, 
                              float2 *minmax, int grid, cudaStream_t st) {
   return launch_checked(k_score_mat<kScoreCPT>, dim3(grid), dim3(kScoreThreads), kSmemBudget, st,
                         packed, evaluated, N, pack, n_active, D, s, minmax);
-}
-
-void launch_narrow_pack(const uint64_t *packed, int64_t n, const PrepArgs &layout, uint32_t *narrow,
-                        cudaStream_t st) {
-  if (n == 0) return;
-  k_narrow_pack<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(packed, n, layout, narrow);
 }
 
 void launch_predict_full(const uint64_t *packed, int64_t count, const uint8_t *nodes,
