@@ -19,6 +19,7 @@
 #include "device_common.cuh"
 #include "internal.h"
 #include "step_common.cuh"
+#include "draws.cuh"
 #include "otf.cuh"
 
 namespace ktune {
@@ -29,7 +30,7 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr int kOtfCap = 4096;                           // on-the-fly list capacity
 constexpr int kOtfBytes = kOtfCap * 12;                 // (W, ordinal, raw32)
 constexpr int kBScoreSmem = 225 * 1024;                  // dynamic shared memory of k_bscore
-constexpr int kSelB = 256;   // select CTA size (the draws themselves run in warp 0)
+constexpr int kSelB = 512;   // select CTA size: a warp per draw looked ahead
 
 __device__ __forceinline__ uint32_t narrow_word_sd(uint32_t nb, const SearchDev &sd) {
   const int f = nb >> 4, t = nb & 15;
@@ -717,21 +718,16 @@ __device__ __forceinline__ uint64_t packed_of_raw(const SearchDev &sd, int64_t r
   return p;
 }
 
-constexpr int kSubCache = 4096;   // sub-tile sums held in shared memory when they fit
-
 __global__ void __launch_bounds__(kSelB) k_bselect(const SearchDev *__restrict__ srch,
                                                   const StepDev *__restrict__ steps) {
-  extern __shared__ __align__(16) uint64_t sel_sm[];
+  extern __shared__ __align__(16) uint8_t sel_sm[];   // kDrawSmem bytes (draws)
   pdl_wait();                 // the weights and their tile sums (or the top-k candidates)
   pdl_launch_dependents();
-  uint64_t *super_sum = sel_sm;                   // [kMaxSuper]
-  uint64_t *sub_c = sel_sm + kMaxSuper;           // [kSubCache]
   __shared__ uint64_t sh64[32];
   __shared__ int64_t pick[KTUNE_MAX_K];
   __shared__ int64_t pick_raw[KTUNE_MAX_K];
   __shared__ float pick_s[KTUNE_MAX_K];
-  __shared__ int64_t sh_sp, sh_sub, sh_l;
-  __shared__ uint64_t sh_r;
+  __shared__ int64_t sh_l;
   const SearchDev &sd = srch[blockIdx.x];
   const StepDev &st = steps[blockIdx.x];
   const int k = st.k;
@@ -787,128 +783,7 @@ __global__ void __launch_bounds__(kSelB) k_bselect(const SearchDev *__restrict__
       ++count;
     }
   } else {
-    // super-tile sums (and the sub-tile sums when they fit in shared memory),
-    // then the k draws by warp 0 alone: super -> sub-tile -> configuration,
-    // each level a warp scan; the chosen sub-tile's 1024 weights are
-    // recomputed from the scores (a configuration drawn earlier in the step
-    // is marked evaluated, so its weight is 0).
-    const int64_t n_sub = (sd.N + kSubTile - 1) / kSubTile;
-    const int64_t n_super = (n_sub + kSuper - 1) / kSuper;
-    const bool cached = n_sub <= kSubCache;
-    uint64_t *subs = cached ? sub_c : sd.sub_sum;
-    for (int64_t sp = threadIdx.x; sp < n_super; sp += blockDim.x) cp_async8(super_sum + sp, sd.super_sum + sp);
-    if (cached)
-      for (int64_t g = threadIdx.x; g < n_sub; g += blockDim.x) cp_async8(sub_c + g, sd.sub_sum + g);
-    cp_async_wait_all();
-    __syncthreads();
-    if (warp == 0) {
-      // descriptor fields in registers: the loop's stores cannot alias them
-      const int64_t N = sd.N;
-      uint32_t *__restrict__ wp = sd.w;
-      uint32_t *__restrict__ evp = sd.eval;
-      uint64_t *__restrict__ subp = sd.sub_sum;
-      const uint64_t seed = sd.seed;
-      const uint32_t sid = sd.search_id, stp = st.step;
-      const int64_t per = (n_super + 31) / 32;
-      const int64_t slo = min(n_super, per * lane), shi = min(n_super, slo + per);
-      // the draws' Philox variates, one lane each, before the serial loop
-      const uint64_t u_lo = philox_u64(seed, sid, stp, (uint32_t)lane, 0u);
-      const uint64_t u_hi = lane + 32 < k ? philox_u64(seed, sid, stp, (uint32_t)(lane + 32), 0u) : 0ull;
-      for (int j = 0; j < k; ++j) {
-        uint64_t local = 0;
-        for (int64_t sp = slo; sp < shi; ++sp) local += super_sum[sp];
-        const uint64_t incl = warp_incl(local);
-        const uint64_t W = __shfl_sync(FULL, incl, 31);
-        if (W == 0) break;
-        const uint64_t uj = j < 32 ? __shfl_sync(FULL, u_lo, j) : __shfl_sync(FULL, u_hi, j - 32);
-        const uint64_t r = scaled_draw(uj, W);
-        // super-tile holding r
-        int64_t sp_sel = -1;
-        uint64_t r1 = 0;
-        if (incl - local <= r && r < incl) {
-          uint64_t acc = incl - local;
-          for (int64_t sp = slo; sp < shi; ++sp) {
-            if (r < acc + super_sum[sp]) {
-              sp_sel = sp;
-              r1 = r - acc;
-              break;
-            }
-            acc += super_sum[sp];
-          }
-        }
-        const int src1 = __ffs(__ballot_sync(FULL, sp_sel >= 0)) - 1;
-        if (src1 < 0) break;   // cannot happen with consistent sums; never index with it
-        sp_sel = __shfl_sync(FULL, sp_sel, src1);
-        r1 = __shfl_sync(FULL, r1, src1);
-        // sub-tile holding r1
-        const int64_t gl = sp_sel * kSuper + lane;
-        const uint64_t v = gl < n_sub ? (cached ? sub_c[gl] : __ldcg(subp + gl)) : 0ull;
-        const uint64_t inc = warp_incl(v);
-        const unsigned hit = __ballot_sync(FULL, inc - v <= r1 && r1 < inc);
-        const int src2 = __ffs(hit) - 1;
-        if (src2 < 0) break;
-        const int64_t g = __shfl_sync(FULL, gl, src2);
-        if (g < 0 || g >= n_sub) break;
-        const uint64_t vg = __shfl_sync(FULL, v, src2);
-        const uint64_t r2 = r1 - __shfl_sync(FULL, inc - v, src2);
-        // configuration holding r2: lane takes 32 consecutive stored weights
-        // (read from L2: earlier draws of this step zeroed theirs)
-        const int64_t i0 = g * kSubTile + lane * 32;
-        uint32_t wv[32];
-        if (i0 + 31 < N) {
-          const uint4 *w4 = reinterpret_cast<const uint4 *>(wp + i0);
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const uint4 x = __ldcg(w4 + q);
-            wv[4 * q] = x.x;
-            wv[4 * q + 1] = x.y;
-            wv[4 * q + 2] = x.z;
-            wv[4 * q + 3] = x.w;
-          }
-        } else {
-#pragma unroll
-          for (int q = 0; q < 32; ++q) wv[q] = i0 + q < N ? __ldcg(wp + i0 + q) : 0u;
-        }
-        // the lane's sum as a tree of adds (depth 5, not a chain of 32)
-        uint64_t t16[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) t16[q] = (uint64_t)wv[2 * q] + wv[2 * q + 1];
-#pragma unroll
-        for (int w = 8; w >= 1; w >>= 1)
-#pragma unroll
-          for (int q = 0; q < w; ++q) t16[q] = t16[2 * q] + t16[2 * q + 1];
-        const uint64_t ls = t16[0];
-        const uint64_t inc3 = warp_incl(ls);
-        const bool mine = inc3 - ls <= r2 && r2 < inc3;
-        uint64_t acc = inc3 - ls;
-        int qsel = -1;
-        uint32_t wsel = 0;
-#pragma unroll
-        for (int q = 0; q < 32; ++q) {
-          if (mine && qsel < 0 && r2 < acc + wv[q]) {
-            qsel = q;
-            wsel = wv[q];
-          }
-          acc += wv[q];
-        }
-        if (mine && qsel >= 0) {
-          const int64_t i = i0 + qsel;
-          pick[j] = i;
-          wp[i] = 0;
-          if (cached) sub_c[g] = vg - wsel;
-          else subp[g] = vg - wsel;
-          super_sum[sp_sel] -= wsel;
-          atomicOr(evp + (i >> 5), 1u << (i & 31));
-        }
-        __threadfence_block();
-        __syncwarp();
-        ++count;
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) sh_l = count;
-    __syncthreads();
-    count = (int)sh_l;
+    count = draw_k(sd, st, sel_sm, pick);
     // scores and raw indices of the picks
     if (sd.mode == 2) {
       if ((int)threadIdx.x < count) pick_s[threadIdx.x] = sd.s[pick[threadIdx.x]];
@@ -1048,7 +923,7 @@ void launch_bweights(const SearchDev *srch, const int *sub_search, int64_t n_sub
 }
 
 void launch_bselect(const SearchDev *srch, const StepDev *steps, int S, cudaStream_t st) {
-  constexpr int smem = (kMaxSuper + kSubCache) * 8;
+  constexpr int smem = kDrawSmem;
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_bselect, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
