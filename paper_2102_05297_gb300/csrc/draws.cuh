@@ -10,11 +10,12 @@
 // search of prefix sums that stay as they were made, and all a draw waits for is
 // its predecessors' intervals, which lanes hold in registers.
 //
-// Before the draws, each warp locates one draw as if it were the first and
-// fetches that sub-tile's weights; the true position is then a few weights away,
-// nearly always in the same sub-tile.  What bounds it: the chain of the k draws,
-// about 400 cycles each (with the picks taken off the sums, every draw scanned the
-// three levels again: about 2,500), behind two dependent L2 round trips.
+// Before the draws, each warp locates one draw as if it were the first, fetches
+// that sub-tile's weights and scans the draw's group of 32; the true position is
+// then a few weights away, most often in the same group, nearly always in the same
+// sub-tile.  What bounds it: two dependent L2 round trips and the chain of the k
+// draws (with the picks taken off the sums, every draw searched the three levels
+// again: about 2,500 cycles each).
 #pragma once
 
 #include "step_common.cuh"
@@ -30,10 +31,14 @@ struct DrawShared {
   uint64_t scan[32];
   uint64_t base[kDrawBufs];      // the weight before the sub-tile in a buffer
   uint64_t sum[kDrawBufs];       // and its own
+  uint64_t gbase[kDrawBufs];     // the same of the group looked ahead to
+  uint64_t gsum[kDrawBufs];
+  uint64_t incl[kDrawBufs][32];  // that group's inclusive prefix sums
   uint64_t rb[KTUNE_MAX_K];      // the picks for the next round's look ahead
   uint64_t W;
   uint32_t w[KTUNE_MAX_K];
   int g[kDrawBufs];              // the sub-tile in a buffer (-1: none)
+  int og[kDrawBufs];             // the group in it
   int n;
 };
 constexpr int kDrawSmem =
@@ -169,8 +174,22 @@ __device__ __noinline__ int draw_k(const SearchDev &sd, const StepDev &st, uint8
           const uint32_t c = lane + 32 < count && sh.rb[lane + 32] <= x ? sh.w[lane + 32] : 0u;
           x += warp_sum30(a, c);
         }
-        if (locate(x, g, base, sum)) fetch(b, g);
-        else g = -1;
+        if (locate(x, g, base, sum)) {
+          fetch(b, g);
+          const uint64_t gl = gp[b * 32 + lane];
+          const unsigned over = __ballot_sync(kFullMask, gl > x - base);
+          const int og = over ? __ffs(over) - 1 : 31;
+          const uint64_t end = __shfl_sync(kFullMask, gl, og), before = __shfl_sync(kFullMask, gl, og > 0 ? og - 1 : 0);
+          const uint64_t gb = og > 0 ? before : 0ull;
+          sh.incl[b][lane] = warp_incl((uint64_t)buf[b * kSubTile + og * 32 + lane]);
+          if (lane == 0) {
+            sh.og[b] = og;
+            sh.gbase[b] = base + gb;
+            sh.gsum[b] = end - gb;
+          }
+        } else {
+          g = -1;
+        }
       }
       if (lane == 0) {
         sh.g[b] = g;
@@ -186,40 +205,41 @@ __device__ __noinline__ int draw_k(const SearchDev &sd, const StepDev &st, uint8
         const uint64_t r = scaled_draw(variate(j0 + b), W);
         const uint64_t add = warp_sum30(rb0 <= r ? pw0 : 0u, rb1 <= r ? pw1 : 0u);
         const uint64_t x = r + add;
-        int g = sh.g[b], bsel = b;
-        uint64_t base = sh.base[b], sum = sh.sum[b];
-        if (!(g >= 0 && x >= base && x - base < sum)) {
-          if (!locate(x, g, base, sum)) break;             // cannot happen with consistent sums
-          const unsigned has = __ballot_sync(kFullMask, my_spec == g);
-          bsel = has ? __ffs(has) - 1 : kDrawBufs;
-          if (!has) fetch(kDrawBufs, g);
-        }
-        const uint64_t y = x - base;
-        const uint64_t gl = gp[bsel * 32 + lane];
-        const unsigned over = __ballot_sync(kFullMask, gl > y);
-        if (!over) break;                                  // cannot happen with consistent sums
-        const int og = __ffs(over) - 1;
-        const uint32_t wq = buf[bsel * kSubTile + og * 32 + lane];
-        const uint64_t gend = __shfl_sync(kFullMask, gl, og);
-        const uint64_t before = __shfl_sync(kFullMask, gl, og > 0 ? og - 1 : 0);
-        const uint64_t gbase = og > 0 ? before : 0ull, y3 = y - gbase;
-        // a group's 32 weights (each at most 2^28) sum below 2^32 but in rare
-        // cases: a 32-bit scan then, else a 64-bit one
-        unsigned hit;
-        uint64_t ex;
-        if (gend - gbase < (1ull << 32)) {
-          const uint32_t iq = warp_incl(wq);
-          hit = __ballot_sync(kFullMask, (uint64_t)(iq - wq) <= y3 && y3 < (uint64_t)iq);
-          ex = iq - wq;
+        int g = sh.g[b];
+        uint32_t w;
+        uint64_t at;
+        int qs, og = sh.og[b];
+        const uint64_t y0 = x - sh.gbase[b];
+        if (g >= 0 && x >= sh.gbase[b] && y0 < sh.gsum[b]) {      // in the group looked ahead to
+          const uint32_t wq = buf[b * kSubTile + og * 32 + lane];
+          const uint64_t iq = sh.incl[b][lane];
+          qs = __ffs(__ballot_sync(kFullMask, iq > y0)) - 1;
+          w = __shfl_sync(kFullMask, wq, qs);
+          at = sh.gbase[b] + __shfl_sync(kFullMask, iq, qs) - w;
         } else {
+          int bsel = b;
+          uint64_t base = sh.base[b], sum = sh.sum[b];
+          if (!(g >= 0 && x >= base && x - base < sum)) {
+            if (!locate(x, g, base, sum)) break;           // cannot happen with consistent sums
+            const unsigned has = __ballot_sync(kFullMask, my_spec == g);
+            bsel = has ? __ffs(has) - 1 : kDrawBufs;
+            if (!has) fetch(kDrawBufs, g);
+          }
+          const uint64_t y = x - base;
+          const uint64_t gl = gp[bsel * 32 + lane];
+          const unsigned over = __ballot_sync(kFullMask, gl > y);
+          if (!over) break;                                // cannot happen with consistent sums
+          og = __ffs(over) - 1;
+          const uint32_t wq = buf[bsel * kSubTile + og * 32 + lane];
+          const uint64_t before = __shfl_sync(kFullMask, gl, og > 0 ? og - 1 : 0);
+          const uint64_t gbase = og > 0 ? before : 0ull;
           const uint64_t iq = warp_incl((uint64_t)wq);
-          hit = __ballot_sync(kFullMask, iq - wq <= y3 && y3 < iq);
-          ex = iq - wq;
+          const unsigned hit = __ballot_sync(kFullMask, iq > y - gbase);
+          if (!hit) break;                                 // cannot happen with consistent sums
+          qs = __ffs(hit) - 1;
+          w = __shfl_sync(kFullMask, wq, qs);
+          at = base + gbase + __shfl_sync(kFullMask, iq, qs) - w;
         }
-        if (!hit) break;                                   // cannot happen with consistent sums
-        const int qs = __ffs(hit) - 1;
-        const uint32_t w = __shfl_sync(kFullMask, wq, qs);
-        const uint64_t at = base + gbase + __shfl_sync(kFullMask, ex, qs);
         if (lane == 0) pick[count] = (int64_t)g * kSubTile + og * 32 + qs;
         // the pick's interval: later intervals begin earlier without it
         if (pb0 > at && pw0) rb0 -= w;

@@ -727,6 +727,7 @@ __global__ void __launch_bounds__(kSelB) k_bselect(const SearchDev *__restrict__
   __shared__ int64_t pick[KTUNE_MAX_K];
   __shared__ int64_t pick_raw[KTUNE_MAX_K];
   __shared__ float pick_s[KTUNE_MAX_K];
+  __shared__ uint64_t pick_p[KTUNE_MAX_K];
   __shared__ int64_t sh_l;
   const SearchDev &sd = srch[blockIdx.x];
   const StepDev &st = steps[blockIdx.x];
@@ -800,6 +801,7 @@ __global__ void __launch_bounds__(kSelB) k_bselect(const SearchDev *__restrict__
       for (int q = 0; q < sd.sa.P; ++q) raw += (int64_t)nib64(p, q) * sd.sa.stride[q];
       pick_raw[threadIdx.x] = raw;
       pick_s[threadIdx.x] = sv;
+      pick_p[threadIdx.x] = p;
     }
     __syncthreads();
   }
@@ -808,7 +810,9 @@ __global__ void __launch_bounds__(kSelB) k_bselect(const SearchDev *__restrict__
     if (sd.select == KTUNE_SELECT_TOPK) atomicOr(sd.eval + (pick[j] >> 5), 1u << (pick[j] & 31));
     st.out_raw[j] = pick_raw[j];
     st.out_score[j] = pick_s[j];
-    if (st.out_packed) st.out_packed[j] = packed_of_raw(sd, pick_raw[j]);
+    // (a division per digit only where the packed form is not stored)
+    if (st.out_packed)
+      st.out_packed[j] = sd.select == KTUNE_SELECT_TOPK || sd.mode == 2 ? packed_of_raw(sd, pick_raw[j]) : pick_p[j];
   }
   if (threadIdx.x == 0 && st.n_out) *st.n_out = count;
 }
