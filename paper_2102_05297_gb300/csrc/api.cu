@@ -1269,7 +1269,7 @@ static void launch_step_kernels(ktune_search *h, const StepBatch<1> &sb, cudaStr
   } else {
     launch_bprep(h->d_srch, h->d_steps, sb, 1, m->K, m->D, st);
     mark(1);
-    launch_bscore(h->d_srch, h->d_steps, h->d_items, h->n_items, h->mode,
+    launch_bscore(h->d_srch, h->d_steps, h->d_items, nullptr, h->n_items, h->mode,
                   h->opts.select == KTUNE_SELECT_TOPK, h->grid, st);
   }
   mark(2);
@@ -1812,34 +1812,51 @@ const BatchVariant kBatchVariants[] = {{0, 1}, {0, 4}, {1, 1}, {2, 1}, {2, 4}, {
 constexpr int kNumBatchVariants = sizeof(kBatchVariants) / sizeof(kBatchVariants[0]);
 
 // Work items of the batch: every search's space (ordinals, or raw tiles when on
-// the fly) cut into pieces of about total / (SMs * items_per_cta) units.
+// the fly), one after the other, cut into SMs * items_per_cta bins of equal cost;
+// a bin that ends inside a search leaves the rest to the next one, so a CTA's
+// bin is a run of neighbouring items.  A piece costs its units and, as it has to
+// stage the search's trees, what about kPieceCost of them would.  (Pieces of
+// total / SMs units of every search on its own gave 32 searches 185 items for
+// 152 CTAs, so that some CTAs had two: 191 us; see k_bscore's bins.)
+constexpr int64_t kPieceCost = 1024;
 int batch_items(ktune_batch *b) {
   std::vector<ItemDev> items;
+  std::vector<int> first;
+  const int bins = b->num_sms * b->items_per_cta;
+  const int64_t piece = b->mode == 2 ? 1 : kPieceCost;
   int64_t total = 0;
   for (ktune_search *h : b->s)
-    if (h->model->kind != 2) total += b->mode == 2 ? h->space->n_tiles : h->space->n_valid;
-  const int64_t target =
-      std::max<int64_t>(b->mode == 2 ? 1 : 1024, total / ((int64_t)b->num_sms * b->items_per_cta));
+    if (h->model->kind != 2) total += (b->mode == 2 ? h->space->n_tiles : h->space->n_valid) + piece;
+  // (every bin may start a piece and leave up to a piece's cost unused)
+  const int64_t target = std::max<int64_t>(2 * piece, (total + bins - 1) / bins + 2 * piece);
+  int64_t room = 0;    // left in the current bin
   for (size_t i = 0; i < b->s.size(); ++i) {
     ktune_search *h = b->s[i];
     b->sdh[i].item_begin = (int64_t)items.size();
-    if (h->model->kind == 2) {   // scored by the MLP kernels, no tree-walk items
-      b->sdh[i].item_end = (int64_t)items.size();
-      continue;
-    }
-    const int64_t units = b->mode == 2 ? h->space->n_tiles : h->space->n_valid;
-    const int64_t pieces = std::max<int64_t>(1, (units + target - 1) / target);
-    for (int64_t q = 0; q < pieces; ++q) {
-      ItemDev it{};
-      it.search = (int)i;
-      it.lo = units * q / pieces;
-      it.hi = units * (q + 1) / pieces;
-      if (it.hi > it.lo) items.push_back(it);
+    if (h->model->kind != 2) {   // (those scored by the MLP kernels have no tree-walk items)
+      const int64_t units = b->mode == 2 ? h->space->n_tiles : h->space->n_valid;
+      for (int64_t lo = 0; lo < units;) {
+        if (room <= piece) {
+          first.push_back((int)items.size());
+          room = target;
+        }
+        ItemDev it{};
+        it.search = (int)i;
+        it.lo = lo;
+        it.hi = std::min(units, lo + room - piece);
+        items.push_back(it);
+        room -= it.hi - lo + piece;
+        lo = it.hi;
+      }
     }
     b->sdh[i].item_end = (int64_t)items.size();
   }
+  b->n_bins = (int)first.size();
+  first.push_back((int)items.size());
   b->n_items = (int)items.size();
-  b->grid = std::min<int>(b->n_items, b->num_sms);
+  b->grid = std::min<int>(b->n_bins, b->num_sms);
+  cudaFree(b->d_first);
+  b->d_first = nullptr;
   cudaFree(b->d_items);
   cudaFree(b->d_cand_key);
   cudaFree(b->d_cand_raw);
@@ -1848,7 +1865,7 @@ int batch_items(ktune_batch *b) {
   b->d_cand_raw = nullptr;
   int rc;
   const size_t n_alloc = std::max<size_t>(1, items.size());
-  if ((rc = dalloc(&b->d_items, n_alloc)) || (rc = dalloc(&b->d_cand_key, n_alloc * KTUNE_MAX_K)) ||
+  if ((rc = dalloc(&b->d_items, n_alloc)) || (rc = dalloc(&b->d_first, first.size())) || (rc = dalloc(&b->d_cand_key, n_alloc * KTUNE_MAX_K)) ||
       (rc = dalloc(&b->d_cand_raw, n_alloc * KTUNE_MAX_K)))
     return rc;
   for (size_t i = 0; i < b->s.size(); ++i) {
@@ -1860,6 +1877,8 @@ int batch_items(ktune_batch *b) {
   if (!items.empty())
     CK(cudaMemcpyAsync(b->d_items, items.data(), items.size() * sizeof(ItemDev),
                        cudaMemcpyHostToDevice, b->stream));
+  CK(cudaMemcpyAsync(b->d_first, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice,
+                     b->stream));
   CK(cudaMemcpyAsync(b->d_srch, b->sdh.data(), b->sdh.size() * sizeof(SearchDev),
                      cudaMemcpyHostToDevice, b->stream));
   CK(cudaStreamSynchronize(b->stream));
@@ -1885,10 +1904,11 @@ int batch_fill_steps(ktune_batch *b, const float *const *counters, int k, StepBa
     sp.cprof_packed = h->cprof_packed;
     host_expert(h->model->roles.data(), K, counters[i], h->opts.inst_reaction, h->opts.cores,
                 sp.delta);
-    sp.out_raw = b->d_out_raw + i * KTUNE_MAX_K;
-    sp.out_score = b->d_out_score + i * KTUNE_MAX_K;
-    sp.out_packed = b->d_out_packed + i * KTUNE_MAX_K;
-    sp.n_out = b->d_nout + i;
+    HostOut &ho = b->hout_dev[i];
+    sp.out_raw = ho.raw;
+    sp.out_score = ho.score;
+    sp.out_packed = ho.packed;
+    sp.n_out = &ho.n_out;
     sp.step = h->step_no;
     sp.k = k;
   }
@@ -1898,23 +1918,38 @@ int batch_fill_steps(ktune_batch *b, const float *const *counters, int k, StepBa
 void batch_launch(ktune_batch *b, const StepBatch<kMaxBatch> &sb, cudaStream_t st, bool score_only) {
   const int S = (int)b->s.size();
   launch_bprep<kMaxBatch>(b->d_srch, b->d_steps, sb, S, b->K_max, b->D_max, st);
-  if (b->n_items > 0)
-    launch_bscore(b->d_srch, b->d_steps, b->d_items, b->n_items, b->mode, b->topk, b->grid, st,
-                  b->variant);
-  if (score_only) return;
   // searches scored by the MLP: prediction of c_profile, then the fused
   // tensor-core forward + Eq. score over all of TS (the same kernels as a
-  // single MLP step)
-  for (const auto &g : b->mlp_groups) {
+  // single MLP step).  On a non-default stream the groups are branches beside
+  // the tree searches, so that one group's launches and last tiles run under
+  // another's (and the trees') work.
+  const int branches = score_only || !b->fork ? 0
+                       : (int)std::min<size_t>(ktune_batch::kBranches, b->mlp_groups.size());
+  if (branches) {
+    cudaEventRecord(b->fork, st);
+    for (int q = 0; q < branches; ++q) cudaStreamWaitEvent(b->branch[q], b->fork, 0);
+  }
+  auto group = [&](const ktune_batch::MlpGroup &g, cudaStream_t gs) {
     const ktune_search *h = g.first;
     const MlpDev md = h->model->mlp->dev();
-    const int S = (int)g.members.size();
-    launch_mlp_fwd(0, md, g.d_cprof, S, g.d_pcprof, nullptr, nullptr, nullptr, nullptr,
-                   h->model->mlp->d_status, 1, st);
+    launch_mlp_fwd(0, md, g.d_cprof, (int)g.members.size(), g.d_pcprof, nullptr, nullptr, nullptr, nullptr,
+                   h->model->mlp->d_status, 1, gs);
     launch_mlp_score_shared(md, h->space->d_packed, h->space->n_valid, g.tg,
-                            h->model->mlp->d_status, b->num_sms, st);
+                            h->model->mlp->d_status, b->num_sms, gs);
+  };
+  if (branches)
+    for (size_t q = 0; q < b->mlp_groups.size(); ++q) group(b->mlp_groups[q], b->branch[q % branches]);
+  if (b->n_items > 0)
+    launch_bscore(b->d_srch, b->d_steps, b->d_items, b->d_first, b->n_bins, b->mode, b->topk, b->grid, st,
+                  b->variant);
+  if (score_only) return;
+  if (!branches)
+    for (const auto &g : b->mlp_groups) group(g, st);
+  for (int q = 0; q < branches; ++q) {
+    cudaEventRecord(b->join[q], b->branch[q]);
+    cudaStreamWaitEvent(st, b->join[q], 0);
   }
-  if (!b->topk) launch_bweights(b->d_srch, b->d_sub_search, b->n_sub, st);
+  if (!b->topk) launch_bweights(b->d_srch, b->d_sub_search, b->n_sub, st, branches == 0);
   launch_bselect(b->d_srch, b->d_steps, S, st);
 }
 
@@ -2006,17 +2041,28 @@ int ktune_batch_create(ktune_search *const *searches, int n, void *stream, ktune
     }
   }
   if ((rc = dalloc(&b->d_srch, n)) || (rc = dalloc(&b->d_steps, n)) ||
-      (rc = dalloc(&b->d_sub_search, sub_search.size())) ||
-      (rc = dalloc(&b->d_out_raw, (size_t)n * KTUNE_MAX_K)) ||
-      (rc = dalloc(&b->d_out_score, (size_t)n * KTUNE_MAX_K)) ||
-      (rc = dalloc(&b->d_out_packed, (size_t)n * KTUNE_MAX_K)) || (rc = dalloc(&b->d_nout, n)))
+      (rc = dalloc(&b->d_sub_search, sub_search.size())))
     return fail(rc);
-  if (cudaMallocHost((void **)&b->h_out_raw, (size_t)n * KTUNE_MAX_K * 8) != cudaSuccess ||
-      cudaMallocHost((void **)&b->h_out_score, (size_t)n * KTUNE_MAX_K * 4) != cudaSuccess ||
-      cudaMallocHost((void **)&b->h_out_packed, (size_t)n * KTUNE_MAX_K * 8) != cudaSuccess ||
-      cudaMallocHost((void **)&b->h_nout, (size_t)n * 4) != cudaSuccess) {
+  if (cudaHostAlloc((void **)&b->hout, (size_t)n * sizeof(HostOut), cudaHostAllocMapped) != cudaSuccess ||
+      cudaMallocHost((void **)&b->h_status, (size_t)std::max<size_t>(1, b->mlp_groups.size()) * sizeof(int)) !=
+          cudaSuccess) {
     set_error("pinned host allocation failed");
     return fail(KTUNE_ENOMEM);
+  }
+  if (cudaHostGetDevicePointer((void **)&b->hout_dev, b->hout, 0) != cudaSuccess) {
+    set_error("mapped host memory is not addressable by the device");
+    return fail(KTUNE_ECUDA);
+  }
+  memset(b->hout, 0, (size_t)n * sizeof(HostOut));
+  if (b->stream && !b->mlp_groups.empty()) {
+    bool ok = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
+    for (int q = 0; q < ktune_batch::kBranches && ok; ++q)
+      ok = cudaStreamCreateWithFlags(&b->branch[q], cudaStreamNonBlocking) == cudaSuccess &&
+           cudaEventCreateWithFlags(&b->join[q], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
+      set_error("branch streams");
+      return fail(KTUNE_ECUDA);
+    }
   }
   if (cudaMemcpyAsync(b->d_sub_search, sub_search.data(), sub_search.size() * 4,
                       cudaMemcpyHostToDevice, b->stream) != cudaSuccess) {
@@ -2030,11 +2076,15 @@ int ktune_batch_create(ktune_search *const *searches, int n, void *stream, ktune
 
 int ktune_batch_destroy(ktune_batch *b) {
   if (!b) return KTUNE_OK;
-  void *dev[] = {b->d_srch, b->d_steps, b->d_items, b->d_sub_search, b->d_cand_key, b->d_cand_raw,
-                 b->d_out_raw, b->d_out_score, b->d_out_packed, b->d_nout};
+  void *dev[] = {b->d_srch, b->d_steps, b->d_items, b->d_first, b->d_sub_search, b->d_cand_key, b->d_cand_raw};
   for (void *p : dev) cudaFree(p);
-  void *pin[] = {b->h_out_raw, b->h_out_score, b->h_out_packed, b->h_nout};
-  for (void *p : pin) cudaFreeHost(p);
+  cudaFreeHost(b->hout);
+  cudaFreeHost(b->h_status);
+  if (b->fork) cudaEventDestroy(b->fork);
+  for (int q = 0; q < ktune_batch::kBranches; ++q) {
+    if (b->join[q]) cudaEventDestroy(b->join[q]);
+    if (b->branch[q]) cudaStreamDestroy(b->branch[q]);
+  }
   for (auto &g : b->mlp_groups) {
     cudaFree(g.d_cprof);
     cudaFree(g.d_pcprof);
@@ -2089,33 +2139,29 @@ int ktune_batch_step(ktune_batch *b, const float *const *counters, int k, int64_
     batch_launch(b, sb, st, false);
   }
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(b->h_out_raw, b->d_out_raw, (size_t)S * KTUNE_MAX_K * 8, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(b->h_out_score, b->d_out_score, (size_t)S * KTUNE_MAX_K * 4, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(b->h_out_packed, b->d_out_packed, (size_t)S * KTUNE_MAX_K * 8, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(b->h_nout, b->d_nout, (size_t)S * 4, cudaMemcpyDeviceToHost, st));
+  // the outputs are in mapped host memory; one status per network comes with them
+  for (size_t q = 0; q < b->mlp_groups.size(); ++q)
+    CK(cudaMemcpyAsync(b->h_status + q, b->mlp_groups[q].first->model->mlp->d_status, sizeof(int),
+                       cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  for (ktune_search *h : b->s)
-    if (h->model->kind == 2) {
-      int status = 0;
-      CK(cudaMemcpy(&status, h->model->mlp->d_status, sizeof(int), cudaMemcpyDeviceToHost));
-      if (status) {
-        cudaMemset(h->model->mlp->d_status, 0, sizeof(int));
-        FAIL(KTUNE_ETIMEOUT, "a tensor-core wait of the MLP timed out");
-      }
+  for (size_t q = 0; q < b->mlp_groups.size(); ++q)
+    if (b->h_status[q]) {
+      cudaMemset(b->mlp_groups[q].first->model->mlp->d_status, 0, sizeof(int));
+      FAIL(KTUNE_ETIMEOUT, "a tensor-core wait of the MLP timed out");
     }
   bool exhausted = false;
   for (int i = 0; i < S; ++i) {
     ktune_search *h = b->s[i];
-    const int no = b->h_nout[i];
+    const HostOut &ho = b->hout[i];
+    const int no = ho.n_out;
     n_out[i] = no;
     exhausted |= no < k;
     for (int j = 0; j < no; ++j) {
-      out_raw[(size_t)i * k + j] = b->h_out_raw[(size_t)i * KTUNE_MAX_K + j];
-      out_score[(size_t)i * k + j] = b->h_out_score[(size_t)i * KTUNE_MAX_K + j];
+      out_raw[(size_t)i * k + j] = ho.raw[j];
+      out_score[(size_t)i * k + j] = ho.score[j];
     }
-    h->last_raw.assign(b->h_out_raw + (size_t)i * KTUNE_MAX_K, b->h_out_raw + (size_t)i * KTUNE_MAX_K + no);
-    h->last_packed.assign(b->h_out_packed + (size_t)i * KTUNE_MAX_K,
-                          b->h_out_packed + (size_t)i * KTUNE_MAX_K + no);
+    h->last_raw.assign(ho.raw, ho.raw + no);
+    h->last_packed.assign(ho.packed, ho.packed + no);
     h->last_scored = h->space->n_valid - h->n_evaluated;
     h->n_evaluated += no;
     h->step_no++;

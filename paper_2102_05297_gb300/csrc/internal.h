@@ -251,10 +251,12 @@ void host_expert(const int *roles, int K, const float *counters, double inst_rea
 int bscore_variants();
 int bscore_variant_threads(int v);
 int bscore_variant_cpt(int v);
-void launch_bscore(const SearchDev *srch, const StepDev *steps, const ItemDev *items, int n_items,
-                   int mode, bool topk, int grid, cudaStream_t st, int variant = 0);
+// first[n_bins + 1]: the items of each bin, one bin after the other per CTA (null: one item per bin)
+void launch_bscore(const SearchDev *srch, const StepDev *steps, const ItemDev *items, const int *first,
+                   int n_bins, int mode, bool topk, int grid, cudaStream_t st, int variant = 0);
+// early: may be scheduled while its predecessor on the stream finishes
 void launch_bweights(const SearchDev *srch, const int *sub_search, int64_t n_sub_total,
-                     cudaStream_t st);
+                     cudaStream_t st, bool early = true);
 void launch_bselect(const SearchDev *srch, const StepDev *steps, int S, cudaStream_t st);
 
 // ---- enumeration (k_space.cu) ----
@@ -515,14 +517,15 @@ struct ktune_batch {
   int *d_sub_search = nullptr;
   uint64_t *d_cand_key = nullptr;
   int64_t *d_cand_raw = nullptr;
-  int64_t *d_out_raw = nullptr;
-  float *d_out_score = nullptr;
-  uint64_t *d_out_packed = nullptr;
-  int *d_nout = nullptr;
-  int64_t *h_out_raw = nullptr;
-  float *h_out_score = nullptr;
-  uint64_t *h_out_packed = nullptr;
-  int *h_nout = nullptr;
+  int *d_first = nullptr;               // the score kernel's bins of items
+  int n_bins = 0;
+  ktune::HostOut *hout = nullptr;       // the searches' outputs, mapped pinned host memory
+  ktune::HostOut *hout_dev = nullptr;
+  int *h_status = nullptr;              // the networks' device-side statuses, pinned
+  // branches of the batched step beside the tree searches: one per MLP group, in turn
+  static constexpr int kBranches = 3;
+  cudaStream_t branch[kBranches] = {};
+  cudaEvent_t fork = nullptr, join[kBranches] = {};
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   cudaGraphNode_t prep_node = nullptr;

@@ -196,7 +196,7 @@ __device__ void topk_merge_cta(uint64_t *lkey, int64_t *lraw, int k, uint64_t *o
 template <int THREADS, int CPT, int MODE, bool TOPK>
 __global__ void __launch_bounds__(THREADS, 1)
     k_bscore(const SearchDev *__restrict__ srch, const StepDev *__restrict__ steps,
-             const ItemDev *__restrict__ items, int n_items) {
+             const ItemDev *__restrict__ items, const int *__restrict__ first, int n_bins) {
   extern __shared__ __align__(16) uint8_t smem[];
   pdl_wait();                 // the prepare kernel's Delta, c_profile and term tables
   pdl_launch_dependents();
@@ -207,7 +207,9 @@ __global__ void __launch_bounds__(THREADS, 1)
   __shared__ int sh_active[KTUNE_MAX_COUNTERS];
   __shared__ int sh_nact;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+  // a CTA's bins of items: bin b holds items first[b] .. first[b + 1) (null: item b)
+  for (int bin = blockIdx.x; bin < n_bins; bin += gridDim.x)
+  for (int item = first ? first[bin] : bin, end = first ? first[bin + 1] : bin + 1; item < end; ++item) {
     const ItemDev it = items[item];
     const SearchDev &sd = srch[it.search];
     const StepDev &st = steps[it.search];
@@ -877,7 +879,7 @@ static void launch_dep(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
 
 template <int THREADS, int CPT, int MODE, bool TOPK>
 static void launch_one(const SearchDev *srch, const StepDev *steps, const ItemDev *items,
-                       int n_items, int grid, cudaStream_t st) {
+                       const int *first, int n_bins, int grid, cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_bscore<THREADS, CPT, MODE, TOPK>,
@@ -885,45 +887,46 @@ static void launch_one(const SearchDev *srch, const StepDev *steps, const ItemDe
     attr = true;
   }
   launch_dep(k_bscore<THREADS, CPT, MODE, TOPK>, dim3(grid), dim3(THREADS), kBScoreSmem, st, srch,
-             steps, items, n_items);
+             steps, items, first, n_bins);
 }
 
 template <int MODE, bool TOPK>
 static void launch_variant(int v, const SearchDev *srch, const StepDev *steps, const ItemDev *items,
-                           int n_items, int grid, cudaStream_t st) {
+                           const int *first, int n_bins, int grid, cudaStream_t st) {
   if constexpr (MODE == 2) {
-    launch_one<512, 4, 2, TOPK>(srch, steps, items, n_items, grid, st);
+    launch_one<512, 4, 2, TOPK>(srch, steps, items, first, n_bins, grid, st);
     return;
   } else {
   switch (v) {
-    case 1: launch_one<512, 4, MODE, TOPK>(srch, steps, items, n_items, grid, st); break;
-    case 2: launch_one<256, 8, MODE, TOPK>(srch, steps, items, n_items, grid, st); break;
-    case 3: launch_one<256, 16, MODE, TOPK>(srch, steps, items, n_items, grid, st); break;
-    case 4: launch_one<384, 8, MODE, TOPK>(srch, steps, items, n_items, grid, st); break;
-    default: launch_one<512, 8, MODE, TOPK>(srch, steps, items, n_items, grid, st);
+    case 1: launch_one<512, 4, MODE, TOPK>(srch, steps, items, first, n_bins, grid, st); break;
+    case 2: launch_one<256, 8, MODE, TOPK>(srch, steps, items, first, n_bins, grid, st); break;
+    case 3: launch_one<256, 16, MODE, TOPK>(srch, steps, items, first, n_bins, grid, st); break;
+    case 4: launch_one<384, 8, MODE, TOPK>(srch, steps, items, first, n_bins, grid, st); break;
+    default: launch_one<512, 8, MODE, TOPK>(srch, steps, items, first, n_bins, grid, st);
   }
   }
 }
 
 // All searches of one launch share the space mode and the select mode.
-void launch_bscore(const SearchDev *srch, const StepDev *steps, const ItemDev *items, int n_items,
+void launch_bscore(const SearchDev *srch, const StepDev *steps, const ItemDev *items, const int *first, int n_bins,
                    int mode, bool topk, int grid, cudaStream_t st, int variant) {
   if (topk) {
-    if (mode == 0) launch_variant<0, true>(variant, srch, steps, items, n_items, grid, st);
-    else if (mode == 1) launch_variant<1, true>(variant, srch, steps, items, n_items, grid, st);
-    else launch_variant<2, true>(variant, srch, steps, items, n_items, grid, st);
+    if (mode == 0) launch_variant<0, true>(variant, srch, steps, items, first, n_bins, grid, st);
+    else if (mode == 1) launch_variant<1, true>(variant, srch, steps, items, first, n_bins, grid, st);
+    else launch_variant<2, true>(variant, srch, steps, items, first, n_bins, grid, st);
   } else {
-    if (mode == 0) launch_variant<0, false>(variant, srch, steps, items, n_items, grid, st);
-    else if (mode == 1) launch_variant<1, false>(variant, srch, steps, items, n_items, grid, st);
-    else launch_variant<2, false>(variant, srch, steps, items, n_items, grid, st);
+    if (mode == 0) launch_variant<0, false>(variant, srch, steps, items, first, n_bins, grid, st);
+    else if (mode == 1) launch_variant<1, false>(variant, srch, steps, items, first, n_bins, grid, st);
+    else launch_variant<2, false>(variant, srch, steps, items, first, n_bins, grid, st);
   }
 }
 
 void launch_bweights(const SearchDev *srch, const int *sub_search, int64_t n_sub_total,
-                     cudaStream_t st) {
+                     cudaStream_t st, bool early) {
   static_assert(kSubTile == 256 * 4, "256 threads x 4 configurations per sub-tile");
-  launch_dep(k_bweights, dim3((unsigned)((n_sub_total + kWSub - 1) / kWSub)), dim3(256), 0, st, srch,
-             sub_search, n_sub_total);
+  const dim3 grid((unsigned)((n_sub_total + kWSub - 1) / kWSub));
+  if (early) launch_dep(k_bweights, grid, dim3(256), 0, st, srch, sub_search, n_sub_total);
+  else k_bweights<<<grid, 256, 0, st>>>(srch, sub_search, n_sub_total);
 }
 
 void launch_bselect(const SearchDev *srch, const StepDev *steps, int S, cudaStream_t st) {
