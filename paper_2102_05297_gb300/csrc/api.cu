@@ -1147,6 +1147,9 @@ int ktune_search_create(ktune_space *s, ktune_model *m, const ktune_search_opts 
     // wins (a CUDA graph on a non-default stream: 40 us per step on the
     // 1,824-configuration space, against 46 us for the cooperative launch)
     h->fused = N >= kFusedDefaultMin ? fshape : 0;
+    // and up to kSmallMax configurations one CTA does the step (while no
+    // per-kernel times are asked for)
+    h->small = h->mode == 0 && o->select == KTUNE_SELECT_SAMPLE && small_step_supported(N, m->D);
   }
   *out = h;
   return KTUNE_OK;
@@ -1348,7 +1351,14 @@ static int enqueue_step(ktune_search *h, const float *counters, int k, int64_t *
   sp.step = h->step_no;
   sp.k = k;
   h->last_fused = h->fused && !h->cached && !h->nbr_radius;
-  if (h->last_fused) {
+  const bool small = h->small && !h->fused && !h->cached && !h->nbr_radius && !h->timing;
+  if (small) {
+    FusedArgs fa{};
+    fa.sd = h->sdh;
+    fa.words = h->d_fz_words;
+    fa.st = sp;
+    CK(launch_step_small(fa, st));
+  } else if (h->last_fused) {
     // one cooperative launch: every CTA of the grid is resident at once
     FusedArgs fa{};
     fa.sd = h->sdh;
@@ -1762,6 +1772,7 @@ int ktune_search_set_fused(ktune_search *h, int shape) {
     FAIL(KTUNE_ESTATE, "on-the-fly spaces take the fused step in shape 2 only");
   CK(cudaStreamSynchronize(h->last_stream));
   h->fused = shape;
+  h->small = false;
   return KTUNE_OK;
 }
 

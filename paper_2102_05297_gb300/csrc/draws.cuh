@@ -44,13 +44,6 @@ struct DrawShared {
 constexpr int kDrawSmem =
     kDrawTop * 8 + (kDrawBufs + 1) * (32 * 8 + kSubTile * 4) + (int)((sizeof(DrawShared) + 15) / 16 * 16);
 
-// Sum over the warp of values below 2^30.
-__device__ __forceinline__ uint64_t warp_sum30(uint32_t a, uint32_t b) {
-  const uint32_t lo = __reduce_add_sync(kFullMask, (a & 0xffffu) + (b & 0xffffu));
-  const uint32_t hi = __reduce_add_sync(kFullMask, (a >> 16) + (b >> 16));
-  return (uint64_t)lo + ((uint64_t)hi << 16);
-}
-
 // Called by the whole CTA; pick[] (shared) receives the ordinals in draw order,
 // the return value is their number.  The picks' weights are zeroed and their
 // evaluated bits set.  smem: kDrawSmem bytes, 16-byte aligned.

@@ -215,6 +215,10 @@ struct FusedArgs {
   uint32_t four;                  // 4, as a launch parameter (the walk's word-offset multiplier)
   StepDev st;
 };
+// The step of a small space as one CTA (k_small.cu).
+constexpr int64_t kSmallMax = 4096;
+bool small_step_supported(int64_t N, int D);
+cudaError_t launch_step_small(const FusedArgs &fa, cudaStream_t st);
 int fused_shapes();
 int fused_blocks_per_sm(int shape);
 int fused_blocks_per_sm_otf();
@@ -580,6 +584,7 @@ struct ktune_search {
   // the whole step as one persistent kernel (tree models, materialised
   // one-word spaces): shape 0 = the four-kernel chain, else fused shape - 1
   int fused = 0;
+  bool small = false;                  // steps as one CTA (k_small.cu), until a shape is asked for
   int fused_grid = 0;
   bool last_fused = false;
   uint32_t *d_fz_words = nullptr;      // [K][L] node words

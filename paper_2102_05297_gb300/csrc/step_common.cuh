@@ -214,6 +214,13 @@ __device__ __forceinline__ T warp_incl(T v) {
   return v;
 }
 
+// Sum over the warp of values below 2^30.
+__device__ __forceinline__ uint64_t warp_sum30(uint32_t a, uint32_t b) {
+  const uint32_t lo = __reduce_add_sync(kFullMask, (a & 0xffffu) + (b & 0xffffu));
+  const uint32_t hi = __reduce_add_sync(kFullMask, (a >> 16) + (b >> 16));
+  return (uint64_t)lo + ((uint64_t)hi << 16);
+}
+
 // Inclusive scan over the block; *total = block sum.  Uses sh[32].
 template <typename T>
 __device__ T block_incl(T v, T *sh, T *total) {
