@@ -399,6 +399,21 @@ void host_expert(const int *roles, int K, const float *cnt, double r, double cor
   }
 }
 
+int host_reacting(const int *roles, int K) {
+  bool seen[KTUNE_PC_N_ROLES] = {false};
+  int n = 0;
+  for (int k = 0; k < K; ++k)
+    switch (roles[k]) {
+      case KTUNE_PC_DRAM_U: case KTUNE_PC_L2_U: case KTUNE_PC_TEX_U: case KTUNE_PC_SHR_U:
+      case KTUNE_PC_INST_EXE: case KTUNE_PC_WARP_E: case KTUNE_PC_WARP_NP_E: case KTUNE_PC_INERT:
+        break;                             // read by the equations, or not at all
+      default:
+        n += !seen[roles[k]];
+        seen[roles[k]] = true;
+    }
+  return n;
+}
+
 }  // namespace ktune
 
 extern "C" {
@@ -1268,7 +1283,7 @@ static void launch_step_kernels(ktune_search *h, const StepBatch<1> &sb, cudaStr
     // least squares: set-up with c_profile's prediction, then predict + score TS
     launch_lsq_prep(h->d_srch, h->d_steps, sb, lsq_pack_bytes(m->lsq_m, m->lsq_nb, m->K), st);
     mark(1);
-    launch_lsq_score(h->d_srch, m->lsq_m, m->lsq_nb, m->K, h->num_sms, st);
+    launch_lsq_score(h->d_srch, m->lsq_m, m->lsq_nb, host_reacting(m->roles.data(), m->K), h->num_sms, st);
   } else {
     launch_bprep(h->d_srch, h->d_steps, sb, 1, m->K, m->D, st);
     mark(1);

@@ -252,6 +252,9 @@ const void *bprep_func();
 // the operation order of the equations; Delta per counter slot as float32.
 void host_expert(const int *roles, int K, const float *counters, double inst_reaction,
                  double cores, float *delta32);
+// Counter slots that a Delta can reach: the first slot of each role that
+// host_expert gives one to.
+int host_reacting(const int *roles, int K);
 int bscore_variants();
 int bscore_variant_threads(int v);
 int bscore_variant_cpt(int v);
@@ -409,7 +412,7 @@ int64_t lsq_pack_bytes(int m, int nb, int K);
 void launch_lsq_prep(const SearchDev *srch, StepDev *steps_dev, const StepBatch<1> &sb,
                      int64_t pack_bytes, cudaStream_t st);
 const void *lsq_prep_func();
-void launch_lsq_score(const SearchDev *srch, int m, int nb, int K, int num_sms, cudaStream_t st);
+void launch_lsq_score(const SearchDev *srch, int m, int nb, int Kr, int num_sms, cudaStream_t st);
 
 // neighbourhood-restricted steps (k_nbr.cu)
 void launch_nbr_step(const SearchDev *srch, StepDev *steps_dev, const StepBatch<1> &sb, int C,

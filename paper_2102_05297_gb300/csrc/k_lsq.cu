@@ -38,17 +38,17 @@ namespace ktune {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int kLsqTile = 4096;         // configurations per sorted tile
+constexpr int kLsqTile = 2048;         // configurations per sorted tile
 constexpr int kLsqSortSubs = 64;       // most subspaces the sorted kernel takes
 constexpr int kLsqSortPack = 160 * 1024;   // largest pack it stages in shared memory
 constexpr int kLsqMaxT = 1 + 2 * KTUNE_MAX_PARAMS + KTUNE_MAX_PARAMS * (KTUNE_MAX_PARAMS - 1) / 2;
 constexpr int kLsqPrepRows = 8192;     // coefficient floats the prepare kernel stages at once
 
-// threads of the sorted kernel: registers grow with m
-template <int M>
-struct SortedShape {
-  static constexpr int threads = 512;
-};
+// Threads of the sorted kernel, two CTAs per SM: while one sorts its tile (loads,
+// histogram, four barriers) the other scores.  2.26M configurations, m = 8, 9
+// active counters: 112 us with one CTA of 512 threads on tiles of 4,096, dealt out
+// whole (3.6 per CTA).
+constexpr int kLsqSortThreads = 256;
 
 __device__ __forceinline__ int okey_l(float f) {
   const int b = __float_as_int(f);
@@ -368,15 +368,16 @@ __global__ void __launch_bounds__(256) k_lsq_prep(const SearchDev *__restrict__ 
 }
 
 template <int M>
-__global__ void __launch_bounds__(SortedShape<M>::threads, 1)
+__global__ void __launch_bounds__(kLsqSortThreads, 2)
     k_lsq_score_s(const SearchDev *__restrict__ srch, int pack_f4) {
   constexpr int T = 1 + 2 * M + M * (M - 1) / 2;
   constexpr int T2 = (T + 1) / 2;
-  constexpr int NT = SortedShape<M>::threads;
+  constexpr int NT = kLsqSortThreads;
   constexpr int CPT = kLsqTile / NT;
   extern __shared__ float4 spack[];
   __shared__ uint64_t s_p[kLsqTile];
-  __shared__ uint16_t s_e[kLsqTile];
+  __shared__ uint32_t s_e[kLsqTile];       // subspace << 16 | place in the tile
+  __shared__ float s_u[KTUNE_MAX_PARAMS * 16];
   __shared__ int hist[kLsqSortSubs + 1], off[kLsqSortSubs + 1];
   __shared__ float sA[KTUNE_MAX_COUNTERS], sD[KTUNE_MAX_COUNTERS];
   __shared__ int s_nact;
@@ -392,18 +393,29 @@ __global__ void __launch_bounds__(SortedShape<M>::threads, 1)
   const int na = s_nact, np = (na + 1) >> 1;
   const int n_f4 = min(pack_f4, n_sub * np * T2);
   for (int i = threadIdx.x; i < n_f4; i += blockDim.x) spack[i] = gpack[i];
-  const uint64_t bmask = q.bmask;
+  for (int i = threadIdx.x; i < KTUNE_MAX_PARAMS * 16; i += NT) s_u[i] = i < sd.sa.P * 16 ? q.utab[i] : 0.0f;
   uint8_t reg[M > 0 ? M : 1];
 #pragma unroll
   for (int a = 0; a < M; ++a) reg[a] = q.reg[a];
-  const float *__restrict__ utab = q.utab;
+  // the subspace's bits: binary parameters (at most 6 here), the first most significant
+  const int nb = q.nb;
+  uint8_t bin[6];
+#pragma unroll
+  for (int b = 0; b < 6; ++b) bin[b] = b < nb ? (uint8_t)(4 * q.bin[b]) : 0;
+  auto sub_of = [&](uint64_t p) {
+    int sub = 0;
+#pragma unroll
+    for (int b = 0; b < 6; ++b)
+      if (b < nb) sub = 2 * sub + (int)((p >> bin[b]) & 1u);
+    return sub;
+  };
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t N = sd.N;
-  const int64_t n_tiles = (N + kLsqTile - 1) / kLsqTile;
+  // this CTA's configurations, an even share of whole words of evaluated bits
+  const int64_t N = sd.N, words = (N + 31) / 32;
+  const int64_t c_lo = words * blockIdx.x / gridDim.x * 32, c_hi = min(N, words * (blockIdx.x + 1) / gridDim.x * 32);
   float mn = FLT_MAX, mx = -FLT_MAX;
   bool any = false;
-  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const int64_t lo = tile * kLsqTile;
+  for (int64_t lo = c_lo; lo < c_hi; lo += kLsqTile) {
     for (int g = threadIdx.x; g <= n_sub; g += NT) hist[g] = 0;
     __syncthreads();          // also orders the pack copy and the previous tile's reads
     uint64_t p[CPT];
@@ -411,8 +423,12 @@ __global__ void __launch_bounds__(SortedShape<M>::threads, 1)
 #pragma unroll
     for (int r = 0; r < CPT; ++r) {
       const int64_t i = lo + r * NT + threadIdx.x;
-      p[r] = i < N ? sd.packed[i] : 0;
-      sub[r] = i < N ? lsq_sub(bmask, p[r]) : n_sub;
+      p[r] = i < c_hi ? __ldg(sd.packed + i) : 0;
+    }
+#pragma unroll
+    for (int r = 0; r < CPT; ++r) {
+      const int64_t i = lo + r * NT + threadIdx.x;
+      sub[r] = i < c_hi ? sub_of(p[r]) : n_sub;
       rank[r] = atomicAdd(&hist[sub[r]], 1);
     }
     __syncthreads();
@@ -435,23 +451,30 @@ __global__ void __launch_bounds__(SortedShape<M>::threads, 1)
     for (int r = 0; r < CPT; ++r) {
       const int at = off[sub[r]] + rank[r];
       s_p[at] = p[r];
-      s_e[at] = (uint16_t)(r * NT + threadIdx.x);
+      s_e[at] = (uint32_t)sub[r] << 16 | (uint32_t)(r * NT + threadIdx.x);
     }
     __syncthreads();
     const int n_in = off[n_sub];
-    // windows of 64 sorted entries: lane takes entries j0 + lane and j0 + 32 + lane
-    for (int j0 = warp * 32 * CPT; j0 < (warp + 1) * 32 * CPT && j0 < n_in; j0 += 64) {
+    // windows of 64 sorted entries, dealt to the warps in turn: lane takes entries
+    // j0 + lane and j0 + 32 + lane
+    for (int j0 = warp * 64; j0 < n_in; j0 += 2 * NT) {
       int jj[2];
       bool in[2];
       int sj[2];
+      uint32_t ej[2];
       uint64_t U[2][M > 0 ? M : 1];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         jj[h] = j0 + 32 * h + lane;
         in[h] = jj[h] < n_in;
         const uint64_t pj = in[h] ? s_p[jj[h]] : 0;
-        sj[h] = in[h] ? lsq_sub(bmask, pj) : -1;
-        lsq_u<M>(pj, reg, utab, U[h]);
+        ej[h] = in[h] ? s_e[jj[h]] : 0u;
+        sj[h] = in[h] ? (int)(ej[h] >> 16) : -1;
+#pragma unroll
+        for (int a = 0; a < M; ++a) {
+          const float u = s_u[reg[a] * 16 + nib64(pj, reg[a])];
+          U[h][a] = pk(u, u);
+        }
       }
       float sc[2] = {0.0f, 0.0f};
       unsigned pa = __ballot_sync(FULL, in[0]), pb = __ballot_sync(FULL, in[1]);
@@ -470,7 +493,7 @@ __global__ void __launch_bounds__(SortedShape<M>::threads, 1)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         if (!in[h]) continue;
-        const int64_t i = lo + s_e[jj[h]];
+        const int64_t i = lo + (ej[h] & 0xffffu);
         const bool ev = (sd.eval[i >> 5] >> (i & 31)) & 1u;
         sd.s[i] = ev ? 0.0f : sc[h];
         if (!ev) {
@@ -547,8 +570,12 @@ void launch_m(const SearchDev *srch, int64_t pack_bytes, int n_sub, int num_sms,
       cudaFuncSetAttribute(k_lsq_score_s<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLsqSortPack);
       attr = true;
     }
-    cfg.gridDim = dim3((unsigned)num_sms);
-    cfg.blockDim = dim3(SortedShape<M>::threads);
+    // two CTAs share an SM where both packs fit
+    int sorted_per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sorted_per_sm, k_lsq_score_s<M>, kLsqSortThreads,
+                                                  (size_t)pack_bytes);
+    cfg.gridDim = dim3((unsigned)(num_sms * std::max(1, sorted_per_sm)));
+    cfg.blockDim = dim3(kLsqSortThreads);
     cfg.dynamicSmemBytes = (size_t)pack_bytes;
     cudaLaunchKernelEx(&cfg, k_lsq_score_s<M>, srch, (int)(pack_bytes / 16));
     return;
@@ -583,8 +610,9 @@ void launch_lsq_prep(const SearchDev *srch, StepDev *steps_dev, const StepBatch<
 
 const void *lsq_prep_func() { return (const void *)k_lsq_prep; }
 
-void launch_lsq_score(const SearchDev *srch, int m, int nb, int K, int num_sms, cudaStream_t st) {
-  const int64_t pb = lsq_pack_bytes(m, nb, K);
+// Kr: the counters that can react at all (the pack holds active ones only)
+void launch_lsq_score(const SearchDev *srch, int m, int nb, int Kr, int num_sms, cudaStream_t st) {
+  const int64_t pb = std::max<int64_t>(16, lsq_pack_bytes(m, nb, Kr));
   const int n_sub = 1 << nb;
   cudaLaunchConfig_t cfg = {};
   cfg.stream = st;
