@@ -319,7 +319,6 @@ __host__ __device__ inline int mlp_n4(int K) { return (K + 31) & ~31; }
 // The network as the fused forward kernel reads it (all device pointers).
 struct MlpDev {
   int P, F, K, Kp;          // parameters, feature columns, counters, counters padded to 16
-  const uint16_t *w[4];     // bf16 row-major: 256 x F, 256 x 256, 256 x 256, Kp x 256
   const float *b[4];        // float32 biases (b[3] padded to Kp)
   const float *range;       // [K] output scale per counter
   const int *off;           // [P + 1] one-hot offset per parameter; off[P] = start of the u block
@@ -341,11 +340,11 @@ struct TrainDev {               // rows: forward, loss gradient, backward
   const float *target;          // counters / range, [n][K]
   const int *off;
   const uint16_t *utab;
-  const uint16_t *w[4], *wt[4]; // bf16 weights and transposes
+  const uint16_t *w[4], *wt[4]; // bf16 weights and transposes, operand layout
   const float *b[4];
   uint16_t *xt, *at[3];         // transposes of the layers' inputs: [F][B], [256][B]
   uint16_t *gzt[3], *gbt;       // transposes of the output gradients: [256][B], [Kp][B]
-  float *gz[3], *g;             // and in float32, [B][256], [B][Kp]
+  float *gz[3], *g;             // and in float32, the same shapes
   double *loss;                 // sum of squared errors, added
   int *status;
 };
@@ -354,7 +353,7 @@ struct WgradDev {               // weight gradients M x N over B rows, and colum
   const uint16_t *A[4], *X[4];  // [M][B], [N][B]
   int M[4], N[4], tiles[4];
   float *ws[4];                 // [splits][M][N]
-  const float *c_src[4];        // [B][c_cols]
+  const float *c_src[4];        // [c_cols][B]
   int c_cols[4];
   float *c_part[4];             // [row blocks][c_cols]
   int *status;
@@ -640,7 +639,7 @@ struct ktune_mlp {
   // float32 master parameters, gradients and Adam moments, 8 tensors:
   // W1 256 x F, b1, W2 256 x 256, b2, W3, b3, W4 Kp x 256 (rows >= K zero), b4 [Kp]
   float *d_p[8] = {}, *d_g[8] = {}, *d_m[8] = {}, *d_v[8] = {};
-  uint16_t *d_wb[4] = {}, *d_wt[4] = {};   // bf16 copies and transposes (d_wt[0] unused)
+  uint16_t *d_wb[4] = {}, *d_wt[4] = {};   // bf16 copies and transposes, operand layout (d_wt[0] unused)
   uint8_t *d_wc = nullptr;                 // chunked operand-layout copy of d_wb
   uint32_t wc_off[4] = {};
   float *d_range = nullptr;

@@ -142,17 +142,16 @@ __global__ void __launch_bounds__(128, 1)
   if (warp == 0) tc::tmem_dealloc(tmem, 256);
 }
 
-// bf16 copy (and optional transpose) of float32 parameters.
+// bf16 copy (and optional transpose) of float32 parameters in the tensor cores'
+// operand layout (core matrices over the whole matrix, KC = its row length).
 __global__ void k_to_bf16(const float *__restrict__ p, int rows, int cols,
                           uint16_t *__restrict__ wb, uint16_t *__restrict__ wt) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= (int64_t)rows * cols) return;
   const uint16_t h = tc::f2bf(p[i]);
-  if (wb) wb[i] = h;
-  if (wt) {
-    const int r = (int)(i / cols), c = (int)(i - (int64_t)r * cols);
-    wt[(size_t)c * rows + r] = h;
-  }
+  const int r = (int)(i / cols), c = (int)(i - (int64_t)r * cols);
+  wb[tc::core_off(r, c, cols) >> 1] = h;
+  if (wt) wt[tc::core_off(c, r, rows) >> 1] = h;
 }
 
 // Per-step set-up of a search scored by the MLP (one CTA): publish the step's

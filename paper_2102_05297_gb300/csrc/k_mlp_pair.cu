@@ -572,7 +572,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   if (warp == 1) tc::tmem_dealloc2(tmem, 512);
 }
 
-// Row-major bf16 weights of the four layers into the chunked operand layout:
+// The four layers' bf16 weights (whole-layer operand layout) into the chunked one:
 // chunk c of a layer holds columns [64 c, 64 c + kc) (the output layer: all 256)
 // of every output row as core matrices with KC = kc, so each CTA's half of the rows is contiguous.
 // One thread moves 8 consecutive columns; the output layer's rows are padded
@@ -590,7 +590,7 @@ __global__ void k_pack_wc(const __grid_constant__ PackArgs pa, uint8_t *__restri
   const int r = p / per_row, k = (p - r * per_row) * 8;
   const int step = mlp_chunk_k(l), c = k / step, kk = k - c * step;
   const int kc = min(step, Kl - c * step);
-  const uint4 v = r < pa.rows[l] ? *reinterpret_cast<const uint4 *>(pa.w[l] + (size_t)r * Kl + k)
+  const uint4 v = r < pa.rows[l] ? *reinterpret_cast<const uint4 *>(pa.w[l] + (tc::core_off(r, k, Kl) >> 1))
                                  : make_uint4(0, 0, 0, 0);
   *reinterpret_cast<uint4 *>(dst + pa.dst[l] + (size_t)c * Nl * step * 2 + tc::core_off(r, kk, kc)) = v;
 }

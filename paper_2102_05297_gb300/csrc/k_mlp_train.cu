@@ -65,59 +65,63 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) 
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-// Rows x Kd bf16 (row-major, leading dimension ld) into core matrices with KC = Kd.
-__device__ __forceinline__ void load_rows(uint8_t *dst, const uint16_t *src, int ld, int rows, int Kd) {
-  const int per_row = Kd >> 3, pieces = rows * per_row;
-  for (int p = threadIdx.x; p < pieces; p += blockDim.x) {
-    const int r = p / per_row, kb = p - r * per_row;
-    cp_async16(dst + tc::core_off(r, kb * 8, Kd), src + (size_t)r * ld + kb * 8);
-  }
-}
-
 __device__ __forceinline__ void tmem_ld1(uint32_t taddr, float &v) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=f"(v) : "r"(taddr));
 }
 
-__device__ __forceinline__ void st_cluster16(uint32_t addr, const uint4 &v) {
-  asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y),
-               "r"(v.z), "r"(v.w)
-               : "memory");
+// Bulk copies with completion on an mbarrier: global to this CTA, and this CTA's
+// shared memory to another CTA of the cluster (dst and bar mapped there).
+__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint64_t *bar) {
+  const uint32_t b = tc::smem_u32(bar);
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(b) : "memory");
+}
+__device__ __forceinline__ void bulk_s2c(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
 __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1)
     k_train_rows(const __grid_constant__ TrainDev td) {
   extern __shared__ __align__(1024) uint8_t sm[];
-  __shared__ uint64_t mbar;
+  // completion of MMAs; weights in buffer s; the other CTAs' activations (exchanges in
+  // turn); the other CTAs are done with the output layer's input
+  __shared__ uint64_t mma, w_full[2], a_full[2], freed;
   __shared__ uint32_t tmem_base;
   __shared__ float sh_b[3][kCols], sh_b4[KTUNE_MAX_COUNTERS];
   // a feature column: 4 x parameter (its shift), | 64 for u, 128 for padding; its digit
   __shared__ uint8_t sh_col[kMlpMaxF], sh_dig[kMlpMaxF];
   __shared__ uint16_t sh_utab[KTUNE_MAX_PARAMS * 16];
   __shared__ int sh_off[KTUNE_MAX_PARAMS + 1];
-  uint8_t *const act[2] = {sm, sm + kActBuf};
-  uint8_t *const wb[2] = {sm + 2 * kActBuf, sm + 2 * kActBuf + kWBuf};
+  const uint32_t act0 = tc::smem_u32(sm), wb0 = act0 + 2u * kActBuf;
   const int F = td.F, K = td.K, Kp = td.Kp, B = td.B, H = kMlpHidden;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)tc::cluster_rank(), n0 = rank * kCols;
-  const int row = (warp & 3) * 32 + lane, chunk = 16 * (warp >> 2);   // this thread's row and columns
-  const int b = (int)(blockIdx.x / kSplitN) * kRows + row;            // its batch row
+  const int row = (warp & 3) * 32 + lane, part = warp >> 2, chunk = 16 * part;   // this thread's row and columns
+  const int b = (int)(blockIdx.x / kSplitN) * kRows + row;                       // its batch row
   const bool live = b < B;
   bool ok = true;
-  uint32_t phase = 0;
 
-  // weights of the first two layers on their way
-  load_rows(wb[0], td.w[0] + (size_t)n0 * F, F, kCols, F);
-  cp_async_commit();
-  load_rows(wb[1], td.w[1] + (size_t)n0 * H, H, kCols, H);
-  cp_async_commit();
-  if (warp == 0) tc::tmem_alloc(&tmem_base, 512);
-  if (threadIdx.x == 0) tc::mbar_init(&mbar, 1);
+  if (threadIdx.x == 0) {
+    tc::mbar_init(&mma, 1);
+    for (int s = 0; s < 2; ++s) {
+      tc::mbar_init(&w_full[s], 1);
+      tc::mbar_init(&a_full[s], 1);
+    }
+    tc::mbar_init(&freed, kSplitN - 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // weights of the first two layers on their way (operand layout: 64 rows are contiguous)
+    bulk_g2s(wb0, td.w[0] + (size_t)n0 * F, (uint32_t)(kCols * F * 2), &w_full[0]);
+    bulk_g2s(wb0 + kWBuf, td.w[1] + (size_t)n0 * H, (uint32_t)(kCols * H * 2), &w_full[1]);
+  }
+  if (warp == 1) tc::tmem_alloc(&tmem_base, 512);
+  const int src = live ? td.idx[b] : 0;
+  const uint64_t pk = live ? td.data[src] : 0ull;
   for (int i = threadIdx.x; i < 3 * kCols; i += blockDim.x) sh_b[i / kCols][i % kCols] = td.b[i / kCols][n0 + i % kCols];
   for (int i = threadIdx.x; i < Kp; i += blockDim.x) sh_b4[i] = td.b[3][i];
   for (int i = threadIdx.x; i <= td.P; i += blockDim.x) sh_off[i] = td.off[i];
   for (int i = threadIdx.x; i < td.P * 16; i += blockDim.x) sh_utab[i] = td.utab[i];
-  const int src = live ? td.idx[b] : 0;
-  const uint64_t pk = live ? td.data[src] : 0ull;
   __syncthreads();
   for (int c = threadIdx.x; c < F; c += blockDim.x) {
     int j = 0;
@@ -129,7 +133,7 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
   __syncthreads();
   // features: one-hot digits, u per parameter, zeros; four threads per row, each CTA
   // of the cluster storing a quarter of the transpose
-  for (int G = warp >> 2; G < F / 8; G += 4) {
+  for (int G = part; G < F / 8; G += 4) {
     uint32_t v[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
@@ -140,49 +144,65 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
     if (live && (G & 3) == rank)
 #pragma unroll
       for (int e = 0; e < 8; ++e) td.xt[(size_t)(8 * G + e) * B + b] = (uint16_t)v[e];
-    *reinterpret_cast<uint4 *>(act[0] + tc::core_off(row, 8 * G, F)) =
+    *reinterpret_cast<uint4 *>(sm + tc::core_off(row, 8 * G, F)) =
         make_uint4(v[0] | v[1] << 16, v[2] | v[3] << 16, v[4] | v[5] << 16, v[6] | v[7] << 16);
   }
+  tc::fence_async_smem();
   tc::fence_before();
   __syncthreads();
   tc::cluster_sync();      // every CTA of the cluster runs: its shared memory may be written
   tc::fence_after();
   const uint32_t tmem = tmem_base, lanes = (uint32_t)((warp & 3) * 32) << 16;
-
-  // D[dcol ..) = act * w^T over Kd columns; returns when it is complete and the
-  // weights of the layer after the next may be loaded into w's buffer
   const bool lead = warp == 0 && tc::elect_one();
-  auto layer = [&](const uint8_t *a, const uint8_t *w, int Kd, int N, uint32_t dcol) {
-    cp_async_wait_group<1>();        // this layer's weights (the next layer's may be in flight)
-    tc::fence_async_smem();
-    __syncthreads();
+  uint32_t n_mma = 0, n_w[2] = {0u, 0u}, n_x = 0;     // phases passed; exchanges begun
+
+  // Layer i of seven (forward 0..3, backward 4..6): D[dcol ..) = a * w^T over Kd columns,
+  // a whole (one KC = Kd buffer) or as the four CTAs' blocks of 64 columns (wait for
+  // exchange x >= 0); then the weights of layer i + 2 go into the buffer that is free.
+  auto layer = [&](int i, uint32_t a, int x, int Kd, int N, uint32_t dcol, const uint16_t *next, int next_bytes) {
+    const int s = i & 1;
     if (warp == 0) {                 // the whole warp, so that descriptors live in uniform registers
-      tc::fence_async_smem();        // what the other CTAs stored, behind the cluster barrier
+      ok = tc::mbar_wait(&w_full[s], n_w[s] & 1u, kTrainWait) && ok;
+      if (x >= 0) ok = tc::mbar_wait(&a_full[x & 1], (uint32_t)(x >> 1) & 1u, kTrainWait) && ok;
+      tc::fence_async_smem();
       tc::fence_after();
       const uint32_t idesc = tc::idesc_bf16(128, N);
-      const uint32_t hi = tc::sdesc_hi((uint32_t)Kd * 16u);
-      uint32_t al = tc::sdesc_lo(tc::smem_u32(a), 128), wl = tc::sdesc_lo(tc::smem_u32(w), 128);
-      for (int k = 0; k < Kd; k += 16, al += 16, wl += 16)   // 256 bytes per step
-        if (lead) tc::mma_bf16(tmem + dcol, tc::sdesc_of(al, hi), tc::sdesc_of(wl, hi), idesc, k ? 1u : 0u);
-      if (lead) tc::mma_commit(&mbar);
+      const uint32_t w_hi = tc::sdesc_hi((uint32_t)Kd * 16u), a_hi = x >= 0 ? tc::sdesc_hi(kCols * 16u) : w_hi;
+      uint32_t wl = tc::sdesc_lo(wb0 + (uint32_t)s * kWBuf, 128);
+      const uint32_t al = tc::sdesc_lo(a, 128);
+      for (int k = 0; k < Kd; k += 16, wl += 16) {           // 256 bytes per step, 16 KB per block of 64 columns
+        const uint32_t ak = x >= 0 ? (uint32_t)((k >> 6) * 1024 + (k & 63)) : (uint32_t)k;
+        if (lead) tc::mma_bf16(tmem + dcol, tc::sdesc_of(al + ak, a_hi), tc::sdesc_of(wl, w_hi), idesc, k ? 1u : 0u);
+      }
+      if (lead) tc::mma_commit(&mma);
       __syncwarp();
     }
-    bool w_ok = tc::mbar_wait(&mbar, phase, kTrainWait);
-    if (!w_ok) w_ok = tc::mbar_wait(&mbar, phase, kTrainWait) && false;   // the MMAs still in flight
+    ++n_w[s];
+    bool w_ok = tc::mbar_wait(&mma, n_mma & 1u, kTrainWait);
+    if (!w_ok) w_ok = tc::mbar_wait(&mma, n_mma & 1u, kTrainWait) && false;   // the MMAs still in flight
+    ++n_mma;
     ok = ok && w_ok;
-    phase ^= 1u;
     tc::fence_after();
+    if (next && threadIdx.x == 0) bulk_g2s(wb0 + (uint32_t)s * kWBuf, next, (uint32_t)next_bytes, &w_full[s]);
   };
-  // 16 bf16 of this thread's row and columns into every CTA's buffer `dst`
-  auto share = [&](uint8_t *dst, const uint32_t (&h)[8]) {
-    const uint4 q0 = make_uint4(h[0], h[1], h[2], h[3]), q1 = make_uint4(h[4], h[5], h[6], h[7]);
-    const uint32_t at = tc::smem_u32(dst) + tc::core_off(row, n0 + chunk, H);
-#pragma unroll
-    for (int r = 0; r < kSplitN; ++r) {
-      const uint32_t p = tc::map_rank(at, (uint32_t)r);
-      st_cluster16(p, q0);
-      st_cluster16(p + 128u, q1);
+  // This thread's 16 bf16 into this CTA's block of buffer `a`, and the block to the others.
+  auto share = [&](uint32_t a, const uint32_t (&h)[8]) {
+    uint8_t *blk = sm + (a - act0) + rank * (kActBuf / kSplitN);
+    *reinterpret_cast<uint4 *>(blk + tc::core_off(row, chunk, kCols)) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4 *>(blk + tc::core_off(row, chunk + 8, kCols)) = make_uint4(h[4], h[5], h[6], h[7]);
+    tc::fence_async_smem();
+    tc::fence_before();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const uint32_t at = a + (uint32_t)rank * (kActBuf / kSplitN), bar = tc::smem_u32(&a_full[n_x & 1]);
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                   "r"((kSplitN - 1) * (kActBuf / kSplitN)) : "memory");
+      for (int r = 1; r < kSplitN; ++r) {
+        const uint32_t to = (uint32_t)((rank + r) & (kSplitN - 1));
+        bulk_s2c(tc::map_rank(at, to), at, kActBuf / kSplitN, tc::map_rank(bar, to));
+      }
     }
+    ++n_x;
   };
   // the same into the transpose [256][B] of a layer
   auto store_t = [&](uint16_t *t, const uint32_t (&h)[8]) {
@@ -191,22 +211,13 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
       for (int i = 0; i < 16; ++i)
         t[(size_t)(n0 + chunk + i) * B + b] = (uint16_t)(i & 1 ? h[i >> 1] >> 16 : h[i >> 1]);
   };
-  auto barrier = [&]() {
-    asm volatile("fence.proxy.async;" ::: "memory");
-    tc::fence_before();
-    __syncwarp();
-    tc::cluster_sync();
-    tc::fence_after();
-  };
 
   // ---- forward: hidden layers 0..2 (accumulators in columns 64 l) ----------------------
 #pragma unroll 1
   for (int l = 0; l < 3; ++l) {
-    layer(act[l & 1], wb[l & 1], l == 0 ? F : H, kCols, (uint32_t)(l * kCols));
-    if (l == 0) load_rows(wb[0], td.w[2] + (size_t)n0 * H, H, kCols, H);
-    else if (l == 1) load_rows(wb[1], td.w[3], H, Kp, H);
-    else load_rows(wb[0], td.wt[3] + (size_t)n0 * Kp, Kp, kCols, Kp);
-    cp_async_commit();
+    layer(l, act0 + (uint32_t)(l & 1) * kActBuf, l - 1, l == 0 ? F : H, kCols, (uint32_t)(l * kCols),
+          l == 0 ? td.w[2] + (size_t)n0 * H : l == 1 ? td.w[3] : td.wt[3] + (size_t)n0 * Kp,
+          l == 0 ? kCols * H * 2 : l == 1 ? Kp * H * 2 : kCols * Kp * 2);
     float v[16], erf[16];
     uint32_t h[8];
     tc::tmem_ld16(tmem + lanes + (uint32_t)(l * kCols + chunk), v);
@@ -218,56 +229,84 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i) h[i] = bf2(v[2 * i], v[2 * i + 1]);
-    share(act[(l + 1) & 1], h);
+    share(act0 + (uint32_t)((l + 1) & 1) * kActBuf, h);
     store_t(td.at[l], h);
     tmem_st16(tmem + lanes + kErfCol + (uint32_t)(l * kCols + chunk), erf);
-    barrier();
   }
-  // ---- output layer (every CTA all of it), loss and its gradient (a quarter of the
-  // columns per CTA, a sixteenth per thread, shared like the activations) --------------
+  // ---- output layer, loss and its gradient: every CTA all of it, a quarter of the columns
+  // per thread; one CTA per quarter adds the errors and stores ---------------------------
   double e = 0.0;
   {
-    const int nc = Kp >> 4, c0 = rank * (Kp >> 2) + (warp >> 2) * nc;
-    float t[4], v[4];
+    const int nc = Kp >> 2, c0 = part * nc;           // 4, 8, 12 or 16 columns
+    const bool mine = part == rank;
+    float t[16], v[16];
+    const float *trow = td.target + (size_t)src * K + c0;
+    const bool vec = (K & 3) == 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      t[i] = i < nc && live && c0 + i < K ? td.target[(size_t)src * K + c0 + i] : 0.0f;
-    layer(act[1], wb[1], H, Kp, kOutCol);
-    load_rows(wb[1], td.wt[2] + (size_t)n0 * H, H, kCols, H);
-    cp_async_commit();
+    for (int i = 0; i < 16; i += 4) {
+      float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (i < nc && live && c0 + i < K) {
+        if (vec) {
+          q = *reinterpret_cast<const float4 *>(trow + i);
+        } else {
+          q.x = trow[i];
+          if (c0 + i + 1 < K) q.y = trow[i + 1];
+          if (c0 + i + 2 < K) q.z = trow[i + 2];
+          if (c0 + i + 3 < K) q.w = trow[i + 3];
+        }
+      }
+      t[i] = q.x;
+      t[i + 1] = q.y;
+      t[i + 2] = q.z;
+      t[i + 3] = q.w;
+    }
+    layer(3, act0 + kActBuf, 2, H, Kp, kOutCol, td.wt[2] + (size_t)n0 * H, kCols * H * 2);
+    if (threadIdx.x == 0)      // the others may write this buffer again
+      for (int r = 1; r < kSplitN; ++r)
+        tc::mbar_arrive_cluster(tc::map_rank(tc::smem_u32(&freed), (uint32_t)((rank + r) & (kSplitN - 1))));
 #pragma unroll
-    for (int i = 0; i < 4; ++i) tmem_ld1(tmem + lanes + kOutCol + (uint32_t)min(c0 + i, Kp - 1), v[i]);
-    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3])::"memory");
+    for (int i = 0; i < 16; ++i) tmem_ld1(tmem + lanes + kOutCol + (uint32_t)min(c0 + i, Kp - 1), v[i]);
+#pragma unroll
+    for (int i = 0; i < 16; i += 4)
+      asm volatile("tcgen05.wait::ld.sync.aligned;"
+                   : "+f"(v[i]), "+f"(v[i + 1]), "+f"(v[i + 2]), "+f"(v[i + 3])::"memory");
     const float bk = (float)B * (float)K;      // below 2^24: exact
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 16; ++i) {
       if (i >= nc) break;
       float g = 0.0f;
       if (live && c0 + i < K) {
         const float d = __fsub_rn(__fadd_rn(v[i], sh_b4[c0 + i]), t[i]);
-        e += (double)d * (double)d;
+        if (mine) e += (double)d * (double)d;
         // 2 d / (B K), one rounding (a float64 quotient rounded to float32 is the same number)
         g = __fdiv_rn(2.0f * d, bk);
       }
-      const uint16_t h = (uint16_t)bf2(g, 0.0f);
-      const uint32_t at = tc::smem_u32(act[0]) + tc::core_off(row, c0 + i, Kp);
+      v[i] = g;
+    }
 #pragma unroll
-      for (int r = 0; r < kSplitN; ++r)
-        asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(tc::map_rank(at, (uint32_t)r)), "h"(h) : "memory");
-      if (live) {
-        td.gbt[(size_t)(c0 + i) * B + b] = h;
-        td.g[(size_t)b * Kp + c0 + i] = g;
+    for (int i = 0; i < 16; i += 4) {
+      if (i >= nc) break;
+      const uint32_t lo = bf2(v[i], v[i + 1]), hi = bf2(v[i + 2], v[i + 3]);
+      *reinterpret_cast<uint2 *>(sm + tc::core_off(row, c0 + i, Kp)) = make_uint2(lo, hi);
+      if (mine && live) {
+        uint16_t *gt = td.gbt + (size_t)(c0 + i) * B + b;
+        gt[0] = (uint16_t)lo;
+        gt[B] = (uint16_t)(lo >> 16);
+        gt[2 * (size_t)B] = (uint16_t)hi;
+        gt[3 * (size_t)B] = (uint16_t)(hi >> 16);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) td.g[(size_t)(c0 + i + q) * B + b] = v[i + q];
       }
     }
-    barrier();
+    tc::fence_async_smem();
+    tc::fence_before();
+    __syncthreads();
   }
   // ---- backward: g_z(l) = (g(l + 1) W(l + 1)) GELU'(z(l)), l = 2, 1, 0 -------------------
 #pragma unroll 1
   for (int l = 2; l >= 0; --l) {
-    const int s = l & 1;                       // l = 2: act[0], wb[0]; 1: act[1], wb[1]; 0: act[0], wb[0]
-    layer(act[s], wb[s], l == 2 ? Kp : H, kCols, kGradCol);
-    if (l == 2) load_rows(wb[0], td.wt[1] + (size_t)n0 * H, H, kCols, H);
-    cp_async_commit();
+    layer(6 - l, act0 + (uint32_t)(l & 1) * kActBuf, l == 2 ? -1 : 4 - l, l == 2 ? Kp : H, kCols, kGradCol,
+          l == 2 ? td.wt[1] + (size_t)n0 * H : nullptr, kCols * H * 2);
     float v[16];
     uint32_t h[8];
     {
@@ -282,22 +321,21 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i) h[i] = bf2(v[2 * i], v[2 * i + 1]);
-    if (l > 0) share(act[s ^ 1], h);
+    if (l == 2) ok = tc::mbar_wait(&freed, 0u, kTrainWait) && ok;
+    if (l > 0) share(act0 + (uint32_t)((l & 1) ^ 1) * kActBuf, h);
+    else tc::fence_before();
     store_t(td.gzt[l], h);
     if (live)
 #pragma unroll
-      for (int i = 0; i < 16; i += 4)
-        *reinterpret_cast<float4 *>(td.gz[l] + (size_t)b * H + n0 + chunk + i) =
-            make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-    if (l > 0) barrier();
+      for (int i = 0; i < 16; ++i) td.gz[l][(size_t)(n0 + chunk + i) * B + b] = v[i];
   }
   for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
   if (lane == 0 && e != 0.0) atomicAdd(td.loss, e);
-  cp_async_wait_all();
-  if (!ok && threadIdx.x == 0) atomicExch(td.status, KTUNE_ETIMEOUT);
+  if (!ok && lane == 0) atomicExch(td.status, KTUNE_ETIMEOUT);
   tc::fence_before();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, 512);
+  tc::cluster_sync();        // the blocks sent from here have arrived
+  if (warp == 1) tc::tmem_dealloc(tmem, 512);
 }
 
 // ---- weight gradients ---------------------------------------------------------------
@@ -328,7 +366,6 @@ __global__ void __launch_bounds__(kWgThreads) k_train_wgrad(const __grid_constan
   extern __shared__ __align__(1024) uint8_t sm[];
   __shared__ uint64_t mbar;
   __shared__ uint32_t tmem_base;
-  __shared__ float part[32][33];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int B = wd.B;
   if ((int)blockIdx.x >= wd.wg_blocks) {
@@ -338,29 +375,27 @@ __global__ void __launch_bounds__(kWgThreads) k_train_wgrad(const __grid_constan
     q /= nb;
     int t = 0;
     while (q >= (wd.c_cols[t] + 31) / 32) q -= (wd.c_cols[t++] + 31) / 32;
-    const int C = wd.c_cols[t], c = q * 32 + lane;
+    const int C = wd.c_cols[t];
     const int r0 = rb * kColRows, r1 = min(B, r0 + kColRows);
-    for (int y = warp; y < 32; y += kWgThreads / 32) {
-      float s = 0.0f;
-      if (c < C)
-        for (int r = r0 + y; r < r1; r += 32) s = __fadd_rn(s, wd.c_src[t][(size_t)r * C + c]);
-      part[y][lane] = s;
-    }
-    __syncthreads();
-    if (warp == 0 && c < C) {
-      float s = 0.0f;
-      for (int y = 0; y < 32; ++y) s = __fadd_rn(s, part[y][lane]);
-      wd.c_part[t][(size_t)rb * C + c] = s;
+    for (int cc = q * 32 + warp; cc < min(C, q * 32 + 32); cc += kWgThreads / 32) {
+      const float *g = wd.c_src[t] + (size_t)cc * B;
+      float s = 0.0f;                          // lane y: rows y, y + 32, ... of the block
+      for (int r = r0 + lane; r < r1; r += 32) s = __fadd_rn(s, g[r]);
+      float sum = 0.0f;
+      for (int y = 0; y < 32; ++y) sum = __fadd_rn(sum, __shfl_sync(0xffffffffu, s, y));
+      if (lane == 0) wd.c_part[t][(size_t)rb * C + cc] = sum;
     }
     return;
   }
   int tile = (int)blockIdx.x / wd.splits, p = 0;
   const int z = (int)blockIdx.x - tile * wd.splits;
   while (tile >= wd.tiles[p]) tile -= wd.tiles[p++];
-  const int M = wd.M[p], N = wd.N[p], nt = (N + kWgTile - 1) / kWgTile;
+  // the accumulator's rows are the weight's columns (the layer's inputs) and its
+  // columns the weight's rows: lanes then store neighbouring addresses
+  const int M = wd.N[p], N = wd.M[p], nt = (N + kWgTile - 1) / kWgTile;
   const int m0 = tile / nt * kWgTile, c0 = tile % nt * kWgTile;
-  const int Nt = min(kWgTile, N - c0), Nm = (Nt + 15) & ~15;
-  const uint16_t *A = wd.A[p] + (size_t)m0 * B, *X = wd.X[p] + (size_t)c0 * B;
+  const int Nt = min(kWgTile, N - c0);
+  const uint16_t *A = wd.X[p] + (size_t)m0 * B, *X = wd.A[p] + (size_t)c0 * B;
   // this slice's rows, in whole chunks of 64
   const int n_chunks = (B + 63) / 64;
   const int lo = (int)((int64_t)n_chunks * z / wd.splits), hi = (int)((int64_t)n_chunks * (z + 1) / wd.splits);
@@ -376,7 +411,7 @@ __global__ void __launch_bounds__(kWgThreads) k_train_wgrad(const __grid_constan
     const int k0 = c * 64, kc = min(64, B - k0);
     uint8_t *s = sm + (c & 1) * kWgStage;
     load_tile(s, A, B, kWgTile, M - m0, k0, kc);
-    load_tile(s + kWgStage / 2, X, B, Nm, Nt, k0, kc);
+    load_tile(s + kWgStage / 2, X, B, Nt, Nt, k0, kc);
     cp_async_commit();
   };
   auto done = [&]() {
@@ -404,7 +439,7 @@ __global__ void __launch_bounds__(kWgThreads) k_train_wgrad(const __grid_constan
     if (threadIdx.x == 0) {
       tc::fence_after();
       const int kc = min(64, B - c * 64);
-      const uint32_t idesc = tc::idesc_bf16(128, Nm), dh = tc::sdesc_hi((uint32_t)kc * 16u);
+      const uint32_t idesc = tc::idesc_bf16(128, Nt), dh = tc::sdesc_hi((uint32_t)kc * 16u);
       const uint32_t s = tc::smem_u32(sm + (c & 1) * kWgStage);
       uint32_t al = tc::sdesc_lo(s, 128), xl = tc::sdesc_lo(s + kWgStage / 2, 128);
       for (int k = 0; k < kc; k += 16, al += 16, xl += 16)
@@ -415,7 +450,7 @@ __global__ void __launch_bounds__(kWgThreads) k_train_wgrad(const __grid_constan
   if (lo < hi) done();
   // slices of fewer rows than 64 x splits may be empty: zeros
   const int row = m0 + (warp & 3) * 32 + lane;
-  float *out = wd.ws[p] + (size_t)z * M * N + (size_t)row * N + c0;
+  float *out = wd.ws[p] + (size_t)z * M * N + (size_t)c0 * M + row;
   for (int c = 16 * (warp >> 2); c < Nt; c += 32) {
     float v[16];
     if (lo < hi) {
@@ -426,8 +461,7 @@ __global__ void __launch_bounds__(kWgThreads) k_train_wgrad(const __grid_constan
     }
     if (row < M)
 #pragma unroll
-      for (int i = 0; i < 16; i += 4)
-        *reinterpret_cast<float4 *>(out + c + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+      for (int i = 0; i < 16; ++i) out[(size_t)(c + i) * M] = v[i];
   }
   if (!ok && threadIdx.x == 0) atomicExch(wd.status, KTUNE_ETIMEOUT);
   tc::fence_before();
@@ -455,12 +489,12 @@ __global__ void __launch_bounds__(256) k_train_update(const __grid_constant__ Up
     const size_t stride = (size_t)ud.rows[t] * ud.cols[t];
     gi = 0.0f;
     int z = 0;
-    for (; z + 8 <= ud.splits; z += 8) {       // eight loads in flight, added in order
-      float v[8];
+    for (; z + 16 <= ud.splits; z += 16) {     // sixteen loads in flight, added in order
+      float v[16];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = w[(size_t)(z + e) * stride];
+      for (int e = 0; e < 16; ++e) v[e] = w[(size_t)(z + e) * stride];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) gi = __fadd_rn(gi, v[e]);
+      for (int e = 0; e < 16; ++e) gi = __fadd_rn(gi, v[e]);
     }
     for (; z < ud.splits; ++z) gi = __fadd_rn(gi, w[(size_t)z * stride]);
   }
@@ -479,11 +513,9 @@ __global__ void __launch_bounds__(256) k_train_update(const __grid_constant__ Up
   ud.p[t][i] = pi;
   if (t & 1) return;
   const uint16_t h = tc::f2bf(pi);
-  ud.wb[t >> 1][i] = h;
-  if (ud.wt[t >> 1]) {
-    const int r = (int)(i / ud.cols[t]), c = (int)(i - (int64_t)r * ud.cols[t]);
-    ud.wt[t >> 1][(size_t)c * ud.rows[t] + r] = h;
-  }
+  const int rows = ud.rows[t], cols = ud.cols[t], r = (int)(i / cols), c = (int)(i - (int64_t)r * cols);
+  ud.wb[t >> 1][tc::core_off(r, c, cols) >> 1] = h;
+  if (ud.wt[t >> 1]) ud.wt[t >> 1][tc::core_off(c, r, rows) >> 1] = h;
 }
 
 }  // namespace

@@ -186,7 +186,6 @@ MlpDev ktune_mlp::dev() const {
   d.K = K;
   d.Kp = Kp;
   for (int l = 0; l < 4; ++l) {
-    d.w[l] = d_wb[l];
     d.b[l] = d_p[2 * l + 1];
   }
   d.range = d_range;
