@@ -658,7 +658,8 @@ struct ktune_mlp {
   uint16_t *d_Xt = nullptr, *d_At[3] = {};   // transposes of the layers' inputs
   float *d_G = nullptr, *d_Gz[3] = {};       // output gradients, float32 and bf16 transposes
   uint16_t *d_Gbt = nullptr, *d_Gzt[3] = {};
-  double *d_loss = nullptr;
+  double *d_loss = nullptr, *d_losses = nullptr;   // of one pass; of each step of a call
+  int cap_losses = 0;
   int *d_status = nullptr;
   float *d_ws = nullptr;                // slices of the weight gradients
   float *d_part = nullptr;              // row blocks of the bias gradients

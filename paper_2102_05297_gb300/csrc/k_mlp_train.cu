@@ -16,9 +16,12 @@
 //   k_train_update the slices summed in a fixed order, and Adam.
 // What bounds it: latency.  The step's arithmetic is 0.4 GFLOP x 9 (about 2 us of
 // tensor work at 4,096 rows); k_train_rows is a chain of seven layers, each an
-// MMA, an epilogue of erff / expf and a cluster barrier.  As 38 launches (one
-// GEMM per layer and direction, transposes, sums and one Adam per tensor) a
-// step took 299 us.
+// MMA, an epilogue of erff / expf and a cluster barrier.  4,096 rows (128
+// CTAs): k_train_rows 36 us, k_train_wgrad 18, k_train_update 6; the update of
+// one step and the rows of the next do not overlap (the weights), the other two
+// launches are scheduled while their predecessor drains (82 -> 77 us per step,
+// 16 steps of 4,096 rows; as 38 launches, one GEMM per layer and direction,
+// transposes, sums and one Adam per tensor, a step took 299 us).
 // Every wait on the tensor cores is bounded: on time-out the kernels record
 // KTUNE_ETIMEOUT, wait once more (bounded) for their MMAs in flight and go on
 // to their end with whatever was computed.
@@ -102,6 +105,7 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
   const int b = (int)(blockIdx.x / kSplitN) * kRows + row;                       // its batch row
   const bool live = b < B;
   bool ok = true;
+  pdl_launch_dependents();
 
   if (threadIdx.x == 0) {
     tc::mbar_init(&mma, 1);
@@ -368,6 +372,8 @@ __global__ void __launch_bounds__(kWgThreads) k_train_wgrad(const __grid_constan
   __shared__ uint32_t tmem_base;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int B = wd.B;
+  pdl_wait();                 // the rows' activations and gradients
+  pdl_launch_dependents();
   if ((int)blockIdx.x >= wd.wg_blocks) {
     int q = (int)blockIdx.x - wd.wg_blocks;
     const int nb = (B + kColRows - 1) / kColRows;
@@ -476,6 +482,7 @@ __global__ void __launch_bounds__(kWgThreads) k_train_wgrad(const __grid_constan
 // the gradient itself.
 __global__ void __launch_bounds__(256) k_train_update(const __grid_constant__ UpdateDev ud) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_wait();                 // the slices and row blocks
   if (i >= ud.total) return;
   int t = 0;
   while (i >= (int64_t)ud.rows[t] * ud.cols[t]) i -= (int64_t)ud.rows[t] * ud.cols[t], ++t;
@@ -518,6 +525,23 @@ __global__ void __launch_bounds__(256) k_train_update(const __grid_constant__ Up
   if (ud.wt[t >> 1]) ud.wt[t >> 1][tc::core_off(c, r, rows) >> 1] = h;
 }
 
+// A launch that may be scheduled while its predecessor finishes; the kernel
+// waits for it in pdl_wait() before touching its results.
+template <typename A>
+void launch_early(void (*kern)(A), int grid, int block, size_t smem, cudaStream_t st, const A &arg) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = st != nullptr ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kern, arg);
+}
+
 }  // namespace
 
 void mlp_train_set_attrs() {
@@ -539,11 +563,11 @@ void launch_train_wgrad(WgradDev wd, cudaStream_t st) {
   }
   wd.wg_blocks = blocks;
   for (int t = 0; t < 4; ++t) blocks += (wd.c_cols[t] + 31) / 32 * train_part_rows(wd.B);
-  k_train_wgrad<<<blocks, kWgThreads, kWgSmem, st>>>(wd);
+  launch_early(k_train_wgrad, blocks, kWgThreads, kWgSmem, st, wd);
 }
 
 void launch_train_update(const UpdateDev &ud, cudaStream_t st) {
-  k_train_update<<<(unsigned)((ud.total + 255) / 256), 256, 0, st>>>(ud);
+  launch_early(k_train_update, (int)((ud.total + 255) / 256), 256, 0, st, ud);
 }
 
 }  // namespace ktune

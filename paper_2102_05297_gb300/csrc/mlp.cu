@@ -338,6 +338,7 @@ int ktune_mlp_destroy(ktune_mlp *m) {
   cudaFree(m->d_G);
   cudaFree(m->d_Gbt);
   cudaFree(m->d_loss);
+  cudaFree(m->d_losses);
   cudaFree(m->d_status);
   cudaFree(m->d_pred_in);
   cudaFree(m->d_pred_out);
@@ -452,10 +453,15 @@ int ktune_mlp_train(ktune_mlp *m, const int32_t *idx, int B, int steps, float lr
   TRY(check_batch(m, B));
   TRY(upload_idx(m, idx, (int64_t)steps * B));
   std::vector<double> sse;
-  double *d_losses = nullptr;
-  if (losses) {
-    TRY(dalloc(&d_losses, (size_t)steps));
-    cudaMemsetAsync(d_losses, 0, (size_t)steps * 8, m->stream);
+  if (losses) {               // kept between calls: an allocation and a free cost as much as two steps
+    if (steps > m->cap_losses) {
+      cudaFree(m->d_losses);
+      m->d_losses = nullptr;
+      m->cap_losses = 0;
+      TRY(dalloc(&m->d_losses, (size_t)steps));
+      m->cap_losses = steps;
+    }
+    cudaMemsetAsync(m->d_losses, 0, (size_t)steps * 8, m->stream);
   }
   const double b1 = 0.9, b2 = 0.999;
   for (int t = 0; t < steps; ++t) {
@@ -469,7 +475,7 @@ int ktune_mlp_train(ktune_mlp *m, const int32_t *idx, int B, int steps, float lr
     a.eps = 1e-8f;
     a.c1 = (float)(1.0 - pow(b1, m->adam_t));
     a.c2 = (float)(1.0 - pow(b2, m->adam_t));
-    enqueue_step(m, m->d_idx + (size_t)t * B, B, losses ? d_losses + t : m->d_loss, &a);
+    enqueue_step(m, m->d_idx + (size_t)t * B, B, losses ? m->d_losses + t : m->d_loss, &a);
   }
   pack_weights(m);
   const cudaError_t le = cudaGetLastError();
@@ -481,14 +487,13 @@ int ktune_mlp_train(ktune_mlp *m, const int32_t *idx, int B, int steps, float lr
   if (losses) {
     if (rc == KTUNE_OK) {
       sse.resize(steps);
-      if (cudaMemcpy(sse.data(), d_losses, (size_t)steps * 8, cudaMemcpyDeviceToHost) != cudaSuccess) {
+      if (cudaMemcpy(sse.data(), m->d_losses, (size_t)steps * 8, cudaMemcpyDeviceToHost) != cudaSuccess) {
         set_error("loss download failed");
         rc = KTUNE_ECUDA;
       } else {
         for (int t = 0; t < steps; ++t) losses[t] = sse[t] / ((double)B * m->K);
       }
     }
-    cudaFree(d_losses);
   }
   return rc;
 }
