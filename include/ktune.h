@@ -310,9 +310,13 @@ int ktune_search_set_neighbourhood(ktune_search *search, int radius);
  * digits by ordinal into a scratch list of N words (so it also writes score 0
  * for the configurations evaluated before the step, which the four kernels
  * leave untouched there), and only shape 2 is offered (others: KTUNE_ESTATE).
- * Shape 2 is the default for the searches it applies to whose TS holds at
- * least 2^18 configurations (smaller ones default to shape 0, whose fixed cost
- * is lower); other searches refuse shapes > 0 (KTUNE_ESTATE).
+ * By default a search that these shapes apply to takes shape 1 (weighted draws,
+ * at most 2,048 configurations per CTA) or shape 2 (others); with at most 4,096
+ * configurations and weighted draws one CTA does the step instead, until this
+ * function is called.  Below 2^18 configurations the default gives way to
+ * shape 0 while per-kernel times are asked for (ktune_search_set_timing), and
+ * on-the-fly spaces default to shape 0.  Other searches refuse shapes > 0
+ * (KTUNE_ESTATE).
  * Cached predictions and neighbourhood-restricted steps keep their own
  * kernels.  Synchronises the search's last stream. */
 int ktune_search_set_fused(ktune_search *search, int shape);

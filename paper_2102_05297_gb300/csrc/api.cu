@@ -1158,13 +1158,21 @@ int ktune_search_create(ktune_space *s, ktune_model *m, const ktune_search_opts 
       set_error("fused-step set-up failed");
       return fail(KTUNE_ECUDA);
     }
-    // below kFusedDefaultMin configurations the four kernels' lower fixed cost
-    // wins (a CUDA graph on a non-default stream: 40 us per step on the
-    // 1,824-configuration space, against 46 us for the cooperative launch)
-    h->fused = N >= kFusedDefaultMin ? fshape : 0;
-    // and up to kSmallMax configurations one CTA does the step (while no
-    // per-kernel times are asked for)
+    // Up to kSmallMax configurations one CTA does the step (while no per-kernel
+    // times are asked for); above, one persistent kernel.  Weighted draws with at
+    // most 2,048 configurations per CTA take 512 threads, whose barriers are
+    // cheaper; from there on 1,024 threads hide more of the walks' latency; the
+    // top-k lists cost the same in both.  us per step, depth-12 trees for 32
+    // counters, 152 CTAs (four kernels as a graph / 512 threads / 1,024): 5,120
+    // configurations 54.3 / 42.4 / 44.9, 163,840 55.4 / 46.0 / 49.8, 262,144
+    // 53.6 / 46.1 / 48.7, 720,896 71.2 / 61.8 / 61.0 (depth 8: 44.4 / 37.6 / 40.6,
+    // 44.8 / 41.1 / 43.0, 44.6 / 41.8 / 43.5, 56.7 / 57.0 / 50.2); top-k, 40
+    // counters: 163,840 71.1 / 47.7 / 46.8.
     h->small = h->mode == 0 && o->select == KTUNE_SELECT_SAMPLE && small_step_supported(N, m->D);
+    const bool few = o->select == KTUNE_SELECT_SAMPLE && N <= (int64_t)2048 * h->fused_grid;
+    if (N >= kFusedDefaultMin || (h->mode == 0 && !h->small))
+      h->fused = !fotf && few && fused_blocks_per_sm(0) >= 1 ? 1 : fshape;
+    h->fused_untimed = N < kFusedDefaultMin;
   }
   *out = h;
   return KTUNE_OK;
@@ -1365,7 +1373,7 @@ static int enqueue_step(ktune_search *h, const float *counters, int k, int64_t *
   sp.n_out = n_out;
   sp.step = h->step_no;
   sp.k = k;
-  h->last_fused = h->fused && !h->cached && !h->nbr_radius;
+  h->last_fused = h->fused && !h->cached && !h->nbr_radius && !(h->fused_untimed && h->timing);
   const bool small = h->small && !h->fused && !h->cached && !h->nbr_radius && !h->timing;
   if (small) {
     FusedArgs fa{};
@@ -1787,7 +1795,7 @@ int ktune_search_set_fused(ktune_search *h, int shape) {
     FAIL(KTUNE_ESTATE, "on-the-fly spaces take the fused step in shape 2 only");
   CK(cudaStreamSynchronize(h->last_stream));
   h->fused = shape;
-  h->small = false;
+  h->small = h->fused_untimed = false;
   return KTUNE_OK;
 }
 

@@ -61,7 +61,10 @@ __host__ __device__ inline int pack_tree_bytes(int D, bool narrow) {
 
 // ---- batched step (k_batch.cu): one launch of each kernel serves S searches ----
 constexpr int kSubTile = 1024;          // configurations per weight sub-tile
-constexpr int64_t kFusedDefaultMin = 1 << 18;   // smallest TS stepped by one persistent kernel by default
+// Spaces below this many configurations keep the four kernels by default where the
+// choice can be seen: while per-kernel times are asked for, and on the fly (whose
+// persistent kernel also writes score 0 for the evaluated configurations).
+constexpr int64_t kFusedDefaultMin = 1 << 18;
 constexpr int kSuper = 32;              // sub-tiles per super-tile (select hierarchy)
 constexpr int kMaxSuper = 4096;         // => at most 134M valid configurations per search
 constexpr int kOtfRun = 4;              // raw indices per thread per decode round (on-the-fly)
@@ -587,6 +590,7 @@ struct ktune_search {
   // one-word spaces): shape 0 = the four-kernel chain, else fused shape - 1
   int fused = 0;
   bool small = false;                  // steps as one CTA (k_small.cu), until a shape is asked for
+  bool fused_untimed = false;          // `fused` holds only while no per-kernel times are asked for
   int fused_grid = 0;
   bool last_fused = false;
   uint32_t *d_fz_words = nullptr;      // [K][L] node words
