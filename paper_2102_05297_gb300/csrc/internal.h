@@ -417,7 +417,7 @@ const void *lsq_prep_func();
 void launch_lsq_score(const SearchDev *srch, int m, int nb, int Kr, int num_sms, cudaStream_t st);
 
 // neighbourhood-restricted steps (k_nbr.cu)
-void launch_nbr_step(const SearchDev *srch, StepDev *steps_dev, const StepBatch<1> &sb, int C,
+void launch_nbr_step(const SearchDev *srch, StepDev *steps_dev, const StepBatch<1> &sb, int C, bool topk,
                      int num_sms, cudaStream_t st);
 const void *nbr_score_func();
 
