@@ -310,8 +310,8 @@ int ktune_search_set_neighbourhood(ktune_search *search, int radius);
  * digits by ordinal into a scratch list of N words (so it also writes score 0
  * for the configurations evaluated before the step, which the four kernels
  * leave untouched there), and only shape 2 is offered (others: KTUNE_ESTATE).
- * By default a search that these shapes apply to takes shape 1 (weighted draws,
- * at most 2,048 configurations per CTA) or shape 2 (others); with at most 4,096
+ * By default a search that these shapes apply to takes shape 1 (at most 4,096
+ * configurations per CTA) or shape 2 (others); with at most 4,096
  * configurations and weighted draws one CTA does the step instead, until this
  * function is called.  Below 2^18 configurations the default gives way to
  * shape 0 while per-kernel times are asked for (ktune_search_set_timing), and

@@ -1158,18 +1158,19 @@ int ktune_search_create(ktune_space *s, ktune_model *m, const ktune_search_opts 
       set_error("fused-step set-up failed");
       return fail(KTUNE_ECUDA);
     }
-    // Up to kSmallMax configurations one CTA does the step (while no per-kernel
-    // times are asked for); above, one persistent kernel.  Weighted draws with at
-    // most 2,048 configurations per CTA take 512 threads, whose barriers are
-    // cheaper; from there on 1,024 threads hide more of the walks' latency; the
-    // top-k lists cost the same in both.  us per step, depth-12 trees for 32
-    // counters, 152 CTAs (four kernels as a graph / 512 threads / 1,024): 5,120
-    // configurations 54.3 / 42.4 / 44.9, 163,840 55.4 / 46.0 / 49.8, 262,144
-    // 53.6 / 46.1 / 48.7, 720,896 71.2 / 61.8 / 61.0 (depth 8: 44.4 / 37.6 / 40.6,
-    // 44.8 / 41.1 / 43.0, 44.6 / 41.8 / 43.5, 56.7 / 57.0 / 50.2); top-k, 40
-    // counters: 163,840 71.1 / 47.7 / 46.8.
+    // Up to kSmallMax configurations (weighted draws) one CTA does the step, while
+    // no per-kernel times are asked for; above, one persistent kernel.  With at most
+    // 4,096 configurations per CTA, one chunk of either shape, it has 512 threads,
+    // whose warps walk only the configurations they have and whose barriers are
+    // cheaper; from there on 1,024 threads hide more of the walks' latency.  us per
+    // step, depth-12 trees for 32 counters, 152 CTAs (four kernels as a graph / 512
+    // threads / 1,024): 5,120 configurations 54.3 / 42.4 / -, 163,840 55.4 / 46.0 /
+    // 53.1, 393,216 55.1 / 52.5 / 54.8, 589,824 - / 52.5 / 55.5, 983,040 - / 64.8 /
+    // 65.8 (depth 8: 44.4 / 37.6 / -, 44.8 / 41.1 / 45.2, 45.1 / 46.6 / 47.4, - /
+    // 48.4 / 47.3, - / 58.0 / 55.1); top-k, 40 counters: 163,840 71.1 / 47.7 / -,
+    // 589,824 - / 59.4 / 60.2, 983,040 - / 74.9 / 72.3.
     h->small = h->mode == 0 && o->select == KTUNE_SELECT_SAMPLE && small_step_supported(N, m->D);
-    const bool few = o->select == KTUNE_SELECT_SAMPLE && N <= (int64_t)2048 * h->fused_grid;
+    const bool few = N <= (int64_t)4096 * h->fused_grid;
     if (N >= kFusedDefaultMin || (h->mode == 0 && !h->small))
       h->fused = !fotf && few && fused_blocks_per_sm(0) >= 1 ? 1 : fshape;
     h->fused_untimed = N < kFusedDefaultMin;
@@ -1852,7 +1853,8 @@ constexpr int kNumBatchVariants = sizeof(kBatchVariants) / sizeof(kBatchVariants
 // bin is a run of neighbouring items.  A piece costs its units and, as it has to
 // stage the search's trees, what about kPieceCost of them would.  (Pieces of
 // total / SMs units of every search on its own gave 32 searches 185 items for
-// 152 CTAs, so that some CTAs had two: 191 us; see k_bscore's bins.)
+// 152 CTAs, so that some CTAs had two: 191 us of score kernel, now 173; see
+// k_bscore's bins.)
 constexpr int64_t kPieceCost = 1024;
 int batch_items(ktune_batch *b) {
   std::vector<ItemDev> items;

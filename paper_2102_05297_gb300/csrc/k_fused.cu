@@ -494,16 +494,21 @@ struct Scorer {
       ev[c] = (last && ok[c]) ? (__ldg(eval_p + (i >> 5)) >> (i & 31)) & 1u : 0u;
     }
     // A warp walks only as many configurations per thread as it has (rounded to
-    // 1, 2, 4, CPT): in a chunk that is not full, a small space's only one, the
+    // 1, 2, 4, 8): in a chunk that is not full, a small space's only one, the
     // other walks would be idle work.  Step of 40,960 configurations, depth-12
-    // trees for 32 counters: 55.0 -> 44.7 us (512 threads x 8), 52.7 -> 47.1
-    // (1,024 x 4); 163,840: 55.6 -> 46.0, 53.1 -> 49.8.
-    const int64_t mine = hi - base - (threadIdx.x & ~31u);
-    const int m = mine <= 0 ? 0 : (int)min((int64_t)CPT, (mine + THREADS - 1) / THREADS);
-    if (m > 4 || CPT <= 2) walk_trees<DT, CPT>(nt, D, L, four, W, s);
-    else if (m > 2) walk_trees<DT, CPT < 4 ? CPT : 4>(nt, D, L, four, W, s);
-    else if (m == 2) walk_trees<DT, CPT < 2 ? CPT : 2>(nt, D, L, four, W, s);
-    else if (m == 1) walk_trees<DT, 1>(nt, D, L, four, W, s);
+    // trees for 32 counters: 55.0 -> 44.7 us; 163,840: 55.6 -> 46.0.  The shapes of
+    // 1,024 threads take spaces whose chunks are nearly full and have no registers
+    // for it (2,257,920 configurations: 89.0 without, 90.2 with).
+    if constexpr (THREADS == 512) {
+      const int64_t mine = hi - base - (threadIdx.x & ~31u);
+      const int m = mine <= 0 ? 0 : (int)min((int64_t)CPT, (mine + THREADS - 1) / THREADS);
+      if (m > 4) walk_trees<DT, CPT>(nt, D, L, four, W, s);
+      else if (m > 2) walk_trees<DT, CPT < 4 ? CPT : 4>(nt, D, L, four, W, s);
+      else if (m == 2) walk_trees<DT, CPT < 2 ? CPT : 2>(nt, D, L, four, W, s);
+      else if (m == 1) walk_trees<DT, 1>(nt, D, L, four, W, s);
+    } else {
+      walk_trees<DT, CPT>(nt, D, L, four, W, s);
+    }
 #pragma unroll
     for (int c = 0; c < CPT; ++c) {
       const int64_t i = base + (int64_t)c * THREADS + threadIdx.x;
