@@ -74,7 +74,7 @@ ALL_PATHS = ("chain", "mlp", "lsq", "cached", "table", "nbr", "batch", "large", 
 PROFILED_TRAFFIC = {
     "k_bscore": 9.637e6,          # profiles/k_bscore_mid_12p.md
     "k_cscore_leaf": 36.564e6,    # profiles/cached_mid_12p.md
-    "k_mlp_pipe": 18.748e6,       # profiles/k_mlp_pipe_mid_12p.md
+    "k_mlp_pair": 18.7e6,         # the packed TS, read once (profiles/k_mlp_pair_mid_12p.md)
     "k_bscore_otf": 20.228e6,     # profiles/k_bscore_otf_large_16p.md
     "k_step_fused": 9.763e6,      # profiles/k_step_fused_mid_12p.md
     "k_step_fused_otf": 378.7e6,  # profiles/k_step_fused_otf_large_16p.md
@@ -556,9 +556,9 @@ def path_mlp(ctx, wl, desc, roles, gpu, sp, valid, digits, tree_model, tree_samp
         "train": {"ms": train_ms, "final_loss": float(losses[-1]), "first_loss": float(losses[0]),
                   "tflops": train_flops / (train_ms / 1e3) / 1e12,
                   "flops": "3 x forward (%d FLOP per row) per row" % fpc},
-        "roofline": {"bound": "tensor", "kernel": "k_mlp_fwd<score> (fused forward + Eq. score)",
+        "roofline": {"bound": "tensor", "kernel": "k_mlp_pair<1> (fused forward + Eq. score)",
                      "achieved": ach / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
-                     "frac": ach / peak, "traffic": PROFILED_TRAFFIC["k_mlp_pipe"],
+                     "frac": ach / peak, "traffic": PROFILED_TRAFFIC["k_mlp_pair"],
                      "peak_source": "%s bf16 burst (cuBLAS GEMM)" % ctx["src"],
                      "flop_per_config": fpc,
                      "kernel_share": {"prepare": kern_ms[0] / kern_ms.sum(),
@@ -1099,7 +1099,7 @@ def path_mlp_large(ctx, n_fit=40000, k=16):
         "speedup_vs_tree": tree_ms / mlp_ms,
         "train": {"ms": train_ms, "final_loss": float(losses[-1]), "first_loss": float(losses[0]),
                   "tflops": 3.0 * fpc * B * steps / (train_ms / 1e3) / 1e12},
-        "roofline": {"bound": "tensor", "kernel": "k_mlp_fwd<score> (fused forward + Eq. score)",
+        "roofline": {"bound": "tensor", "kernel": "k_mlp_pair<1> (fused forward + Eq. score)",
                      "achieved": ach / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
                      "frac": ach / peak, "traffic": None,
                      "peak_source": "%s bf16 burst (cuBLAS GEMM)" % ctx["src"],
@@ -1127,7 +1127,7 @@ def path_tiny(ctx):
             "us_per_step_median": 1e3 * statistics.median(step_ms),
             "us_per_step_mean": 1e3 * sum(step_ms) / n_steps,
             "value": scored / (sum(step_ms) / 1e3), "unit": "configs/s",
-            "bound": "launch latency (one CUDA-graph launch of 4 kernels per step)"}
+            "bound": "latency (one kernel of one CTA per step)"}
 
 
 # ---------------------------------------------------------------------------

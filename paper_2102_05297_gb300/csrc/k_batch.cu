@@ -12,7 +12,7 @@
 //              integer weights, sub-tile sums (weighted-sample searches).
 //   k_bselect  one CTA per search: k draws without replacement over a
 //              super-tile / sub-tile / configuration hierarchy (Section 3.6,
-//              Algorithm 1), or the merge of the top-k candidates.
+//              Algorithm 1; draws.cuh), or the merge of the top-k candidates.
 #include <float.h>
 #include <limits.h>
 

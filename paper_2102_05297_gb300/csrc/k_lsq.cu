@@ -46,7 +46,7 @@ constexpr int kLsqPrepRows = 8192;     // coefficient floats the prepare kernel 
 
 // Threads of the sorted kernel, two CTAs per SM: while one sorts its tile (loads,
 // histogram, four barriers) the other scores.  2.26M configurations, m = 8, 9
-// active counters: 112 us with one CTA of 512 threads on tiles of 4,096, dealt out
+// active counters: 93 us; 112 with one CTA of 512 threads on tiles of 4,096, dealt out
 // whole (3.6 per CTA).
 constexpr int kLsqSortThreads = 256;
 
