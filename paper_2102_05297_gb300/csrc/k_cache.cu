@@ -176,8 +176,8 @@ constexpr int kLeafCols = 4;   // columns read ahead per thread: 32 KB in flight
 // warp-wide load), with the tables' copy in front.  Each CTA has an even share of
 // the groups, and every batch of columns is read while the one before is added,
 // the first while the tables arrive: the cached step of 2,257,920 configurations,
-// depth-12 trees for 32 counters, 69.8 -> 60.8 us (read, then added, 4 columns
-// at a time, this kernel took 32 us of it).
+// depth-12 trees for 32 counters, 69.8 -> 60.8 us (this kernel alone, cold: 32
+// -> 25; before, 4 columns were read, then added).
 __global__ void __launch_bounds__(512, 1)
     k_cscore_leaf(const SearchDev *__restrict__ srch, const uint16_t *__restrict__ leaves,
                   int64_t Np, int tree_bytes, int terms_off, int stage_bytes) {

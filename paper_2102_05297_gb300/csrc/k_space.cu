@@ -13,8 +13,9 @@
 // run's 16 valid bits (raw size / 8 bytes), so that the writing pass decodes
 // only runs that hold a valid configuration.  What bounds the counting pass is
 // the instructions per raw index (odometer, bit).  41.3M raw, 2.26M valid
-// configurations: 290 + 306 + 12 us with a table load and a digit sum per
-// constraint group in both passes and a third pass for the one-word form.
+// configurations: 105 us counting, 45 writing; 290 + 306 + 12 us with a table
+// load and a digit sum per constraint group in both passes and a third pass for
+// the one-word form.
 #include "internal.h"
 
 namespace ktune {
