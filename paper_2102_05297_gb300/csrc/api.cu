@@ -608,22 +608,55 @@ int ktune_space_decode(const ktune_space *s, int64_t raw, int64_t *values_out) {
 
 // Read-back of a range of TS: from kReadOnDevice configurations on, converted by
 // a kernel into a temporary device buffer and copied straight to the caller
-// (2.26M raw indices: 8.7 ms on one host thread, see ktune_space_valid_raw);
-// below, the packed digits are copied and converted here (a few tens of
-// microseconds, no allocation).
+// (2.26M raw indices: 8.7 ms on one host thread, see ktune_space_valid_raw), at
+// most kReadChunk configurations at a time, so that the buffer stays small
+// beside any space; below, or where not even that buffer is to be had, the packed
+// digits are copied and converted here.  Either way on the space's own device,
+// whichever is current.
 extern "C++" {
 namespace {
 constexpr int64_t kReadOnDevice = 8192;
-template <typename F>
-int read_device(int64_t bytes, void *out, F convert, int64_t out_bytes = -1) {
-  uint8_t *tmp = nullptr;
-  TRY(dalloc(&tmp, (size_t)bytes));
-  convert(tmp);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess)
-    e = cudaMemcpy(out, tmp, out_bytes < 0 ? bytes : out_bytes, cudaMemcpyDeviceToHost);
-  cudaFree(tmp);
-  if (e != cudaSuccess) FAIL(KTUNE_ECUDA, std::string("read-back: ") + cudaGetErrorString(e));
+constexpr int64_t kReadChunk = 1 << 22;       // a multiple of 4: digits are made in whole words
+
+struct OnDevice {
+  int was = -1;
+  explicit OnDevice(int dev) {
+    if (cudaGetDevice(&was) == cudaSuccess && was != dev) cudaSetDevice(dev);
+    else was = -1;
+  }
+  ~OnDevice() {
+    if (was >= 0) cudaSetDevice(was);
+  }
+};
+
+// bytes of output per configuration; device(from, n, tmp) enqueues a conversion
+// and host(digits, at) makes one.
+template <typename D, typename H>
+int read_back(const ktune_space *s, int64_t first, int64_t count, int64_t bytes, void *out, D device, H host) {
+  OnDevice on(s->device);
+  uint8_t *dst = static_cast<uint8_t *>(out);
+  if (count >= kReadOnDevice) {
+    uint8_t *tmp = nullptr;
+    if (cudaMalloc((void **)&tmp, (size_t)((std::min(count, kReadChunk) * bytes + 3) / 4 * 4)) == cudaSuccess) {
+      cudaError_t e = cudaSuccess;
+      for (int64_t at = 0; at < count && e == cudaSuccess; at += kReadChunk) {
+        const int64_t n = std::min(count - at, kReadChunk);
+        device(s->d_packed + first + at, n, tmp);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpy(dst + at * bytes, tmp, (size_t)(n * bytes), cudaMemcpyDeviceToHost);
+      }
+      cudaFree(tmp);
+      if (e != cudaSuccess) FAIL(KTUNE_ECUDA, std::string("read-back: ") + cudaGetErrorString(e));
+      return KTUNE_OK;
+    }
+    cudaGetLastError();                       // no room: converted here
+  }
+  std::vector<uint64_t> p((size_t)std::min(count, kReadChunk));
+  for (int64_t at = 0; at < count; at += kReadChunk) {
+    const int64_t n = std::min(count - at, kReadChunk);
+    CK(cudaMemcpy(p.data(), s->d_packed + first + at, (size_t)n * 8, cudaMemcpyDeviceToHost));
+    for (int64_t i = 0; i < n; ++i) host(p[(size_t)i], at + i);
+  }
   return KTUNE_OK;
 }
 }  // namespace
@@ -633,36 +666,31 @@ int ktune_space_valid_raw(const ktune_space *s, int64_t first, int64_t count, in
   if (!s || (!out_raw && count)) FAIL(KTUNE_EINVAL, "null argument");
   if (!s->d_packed) FAIL(KTUNE_ESTATE, "space is not materialised");
   if (first < 0 || count < 0 || first + count > s->n_valid) FAIL(KTUNE_EINVAL, "range out of TS");
-  if (count >= kReadOnDevice) {
-    return read_device(count * 8, out_raw, [&](void *tmp) {
-      launch_raw_of(s->d_packed + first, count, s->sa, static_cast<int64_t *>(tmp), nullptr);
-    });
-  }
-  std::vector<uint64_t> p((size_t)count);
-  if (count) CK(cudaMemcpy(p.data(), s->d_packed + first, count * 8, cudaMemcpyDeviceToHost));
-  for (int64_t i = 0; i < count; ++i) {
-    int64_t raw = 0;
-    for (int j = 0; j < s->sa.P; ++j) raw += (int64_t)((p[i] >> (4 * j)) & 15u) * s->sa.stride[j];
-    out_raw[i] = raw;
-  }
-  return KTUNE_OK;
+  return read_back(
+      s, first, count, 8, out_raw,
+      [&](const uint64_t *from, int64_t n, void *tmp) {
+        launch_raw_of(from, n, s->sa, static_cast<int64_t *>(tmp), nullptr);
+      },
+      [&](uint64_t p, int64_t i) {
+        int64_t r = 0;
+        for (int j = 0; j < s->sa.P; ++j) r += (int64_t)((p >> (4 * j)) & 15u) * s->sa.stride[j];
+        out_raw[i] = r;
+      });
 }
 
 int ktune_space_valid_digits(const ktune_space *s, int64_t first, int64_t count, uint8_t *out) {
   if (!s || (!out && count)) FAIL(KTUNE_EINVAL, "null argument");
   if (!s->d_packed) FAIL(KTUNE_ESTATE, "space is not materialised");
   if (first < 0 || count < 0 || first + count > s->n_valid) FAIL(KTUNE_EINVAL, "range out of TS");
-  if (count >= kReadOnDevice) {
-    return read_device((count * s->sa.P + 3) / 4 * 4, out, [&](void *tmp) {
-      launch_digits_of(s->d_packed + first, count, s->sa.P, static_cast<uint32_t *>(tmp), nullptr);
-    }, count * s->sa.P);
-  }
-  std::vector<uint64_t> p((size_t)count);
-  if (count) CK(cudaMemcpy(p.data(), s->d_packed + first, count * 8, cudaMemcpyDeviceToHost));
   const int P = s->sa.P;
-  for (int64_t i = 0; i < count; ++i)
-    for (int j = 0; j < P; ++j) out[i * P + j] = (uint8_t)((p[i] >> (4 * j)) & 15u);
-  return KTUNE_OK;
+  return read_back(
+      s, first, count, P, out,
+      [&](const uint64_t *from, int64_t n, void *tmp) {
+        launch_digits_of(from, n, P, static_cast<uint32_t *>(tmp), nullptr);
+      },
+      [&](uint64_t p, int64_t i) {
+        for (int j = 0; j < P; ++j) out[i * P + j] = (uint8_t)((p >> (4 * j)) & 15u);
+      });
 }
 
 const uint64_t *ktune_space_packed_device(const ktune_space *s) { return s ? s->d_packed : nullptr; }
