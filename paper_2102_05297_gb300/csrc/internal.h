@@ -454,6 +454,7 @@ int dalloc(T **p, size_t n) {
   if (n == 0) n = 1;
   cudaError_t e = cudaMalloc((void **)p, n * sizeof(T));
   if (e != cudaSuccess) {
+    cudaGetLastError();   // reported here: a later call that checks its launches is not to see it
     set_error(std::string("cudaMalloc: ") + cudaGetErrorString(e));
     return KTUNE_ENOMEM;
   }

@@ -62,3 +62,12 @@ def test_read_back_beside_a_full_device(kt, left):
         np.testing.assert_array_equal(sp.valid_digits(), dig)
         np.testing.assert_array_equal(sp.valid_raw(7, n - 8), raw[7:n - 1])
     np.testing.assert_array_equal(dig, np.stack(np.unravel_index(raw, radices), axis=1))
+
+
+def test_failed_allocation_is_reported_once(kt):
+    """A creation that does not fit fails with KTUNE_ENOMEM, and only that one."""
+    with Filled(6 * MB):
+        with pytest.raises(kt.KtuneError, match="cudaMalloc"):
+            make(kt, [16, 16, 16, 16, 16, 5], [])
+        assert make(kt, [3, 5], []).count() == (15, 15)
+    assert make(kt, [3, 5], []).count() == (15, 15)
