@@ -506,40 +506,53 @@ int ktune_space_create(const ktune_space_desc *d, int flags, void *stream, ktune
       return cleanup(KTUNE_ECUDA);
     }
   }
+  s->n_tiles = (s->sa.n_raw + kEnumTileRaw - 1) / kEnumTileRaw;
+  // scratch of the enumeration: the tiles' counts and, for the writing pass of a
+  // materialised space, the runs' valid bits (up to 128 MB; larger raw spaces, and
+  // those for whose bits there is no room, are checked again there)
+  int32_t *d_count = nullptr;
+  uint16_t *d_masks = nullptr;
+  auto drop = [&](auto *&d) {
+    cudaFree(d);
+    d = nullptr;
+  };
+  if ((rc = dalloc(&s->d_tile_offset, s->n_tiles + 1)) || (rc = dalloc(&d_count, s->n_tiles)) ||
+      (s->ci_combos && (rc = dalloc(&s->d_ci_table, (size_t)((s->ci_combos + 31) / 32))))) {
+    drop(d_count);
+    return cleanup(rc);
+  }
+  if (flags == KTUNE_MATERIALISE && s->sa.n_raw <= (int64_t)1 << 30 &&
+      dalloc(&d_masks, (size_t)s->n_tiles * kEnumThreads))
+    d_masks = nullptr;
   CiArgs ci{};
   if (s->ci_combos) {
     ci.words = (int)((s->ci_combos + 31) / 32);
     for (int j = 0; j < s->sa.P; ++j) ci.stride[j] = s->ci_stride[j];
-    if ((rc = dalloc(&s->d_ci_table, ci.words))) return cleanup(rc);
     launch_ci_table(s->sa, s->d_groups, s->d_table, ci, s->ci_combos, s->d_ci_table, cs);
     ci.table = s->d_ci_table;
-  }
-  s->n_tiles = (s->sa.n_raw + kEnumTileRaw - 1) / kEnumTileRaw;
-  // scratch of the enumeration: the tiles' counts and, for the writing pass of a
-  // materialised space, the runs' valid bits (up to 128 MB; larger raw spaces are
-  // checked again there)
-  int32_t *d_count = nullptr;
-  uint16_t *d_masks = nullptr;
-  auto drop = [&]() {
-    cudaFree(d_count);
-    cudaFree(d_masks);
-  };
-  if ((rc = dalloc(&d_count, s->n_tiles)) || (rc = dalloc(&s->d_tile_offset, s->n_tiles + 1)) ||
-      (flags == KTUNE_MATERIALISE && s->sa.n_raw <= (int64_t)1 << 30 &&
-       (rc = dalloc(&d_masks, s->n_tiles * kEnumThreads)))) {
-    drop();
-    return cleanup(rc);
   }
   launch_enum_count(s->sa, s->d_groups, s->d_table, ci, s->n_tiles, d_count, d_masks, cs);
   launch_scan_tiles(d_count, s->n_tiles, s->d_tile_offset, cs);
   cudaError_t e = cudaMemcpyAsync(&s->n_valid, s->d_tile_offset + s->n_tiles, sizeof(int64_t),
                                   cudaMemcpyDeviceToHost, cs);
   if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  drop(d_count);
   if (e == cudaSuccess && flags == KTUNE_MATERIALISE) {
     WordArgs wa{};
     for (int j = 0; j < s->sa.P; ++j) wa.pos[j] = s->pos[j];
-    if ((rc = dalloc(&s->d_packed, s->n_valid)) || (s->narrow && (rc = dalloc(&s->d_narrow, s->n_valid)))) {
-      drop();
+    auto outputs = [&]() -> int {
+      const int r = dalloc(&s->d_packed, s->n_valid);
+      return r || !s->narrow ? r : dalloc(&s->d_narrow, s->n_valid);
+    };
+    rc = outputs();
+    if (rc && d_masks) {            // the bits' room for the configurations themselves
+      drop(d_masks);
+      drop(s->d_packed);
+      rc = outputs();
+    }
+    if (rc) {
+      drop(d_masks);
       return cleanup(rc);
     }
     launch_enum_write(s->sa, s->d_groups, s->d_table, d_masks, s->n_tiles, s->d_tile_offset, s->d_packed,
@@ -547,7 +560,7 @@ int ktune_space_create(const ktune_space_desc *d, int flags, void *stream, ktune
     e = cudaStreamSynchronize(cs);
     if (e == cudaSuccess) e = cudaGetLastError();
   }
-  drop();
+  drop(d_masks);
   if (e != cudaSuccess) {
     set_error(std::string("enumeration: ") + cudaGetErrorString(e));
     return cleanup(KTUNE_ECUDA);

@@ -71,3 +71,20 @@ def test_failed_allocation_is_reported_once(kt):
             make(kt, [16, 16, 16, 16, 16, 5], [])
         assert make(kt, [3, 5], []).count() == (15, 15)
     assert make(kt, [3, 5], []).count() == (15, 15)
+
+
+# 2^30 raw indices, whose valid bits would take 134 MB: no room for them at all
+# (81,920 configurations), or for them but not for 8.1M configurations beside them
+@pytest.mark.parametrize("total,left", [(5, 48 * MB), (12, 160 * MB)])
+def test_creation_without_room_for_the_valid_bits(kt, total, left):
+    radices, code = [16] * 7 + [4], W.c_sum_le([0, 1, 2, 3], total)
+    ref = make(kt, radices, code)
+    raw = ref.valid_raw()
+    ref.close()
+    with Filled(left):
+        sp = make(kt, radices, code)
+        assert sp.count() == (len(raw), 1 << 30)
+        got = sp.valid_raw()
+    np.testing.assert_array_equal(got, raw)
+    digits = np.stack(np.unravel_index(raw[::997], radices), axis=1)
+    assert np.all(digits[:, :4].sum(axis=1) + 4 <= total)
