@@ -313,8 +313,10 @@ int ktune_search_set_neighbourhood(ktune_search *search, int radius);
  * By default a search that these shapes apply to takes shape 1 (at most 4,096
  * configurations per CTA) or shape 2 (others); with at most 4,096
  * configurations and weighted draws one CTA does the step instead, until this
- * function is called.  Below 2^18 configurations the default gives way to
- * shape 0 while per-kernel times are asked for (ktune_search_set_timing), and
+ * function is called.  Below 2^18 configurations the default takes only as many
+ * CTAs as let the steps of several searches run side by side (fewer for
+ * ktune_step_device than for ktune_step), and it gives way to shape 0 while
+ * per-kernel times are asked for (ktune_search_set_timing), and
  * on-the-fly spaces default to shape 0.  Other searches refuse shapes > 0
  * (KTUNE_ESTATE).
  * Cached predictions and neighbourhood-restricted steps keep their own

@@ -1187,13 +1187,13 @@ int ktune_search_create(ktune_space *s, ktune_model *m, const ktune_search_opts 
     const int mm0[2] = {INT_MAX, INT_MIN};
     if ((rc = dalloc(&h->d_fz_words, (size_t)m->K * L)) || (rc = dalloc(&h->d_fz_terms, (size_t)m->K * L)) ||
         (rc = dalloc(&h->d_fz_mm, 2)) || (rc = dalloc(&h->d_fz_phase, 8)) ||
-        (rc = dalloc(&h->d_fz_sync, 2)) || (rc = dalloc(&h->d_fz_status, 1)) ||
+        (rc = dalloc(&h->d_fz_sync, 6)) || (rc = dalloc(&h->d_fz_status, 1)) ||
         (rc = dalloc(&h->d_fz_cand, (size_t)h->fused_grid * KTUNE_MAX_K)) ||
         (fotf && (rc = dalloc(&h->d_fz_list, (size_t)N))))
       return fail(rc);
     if (launch_fused_words(m->d_nodes, m->K, m->D, lay, h->d_fz_words, cs) != cudaSuccess ||
         cudaMemcpyAsync(h->d_fz_mm, mm0, 8, cudaMemcpyHostToDevice, cs) != cudaSuccess ||
-        cudaMemsetAsync(h->d_fz_sync, 0, 16, cs) != cudaSuccess ||
+        cudaMemsetAsync(h->d_fz_sync, 0, 48, cs) != cudaSuccess ||
         cudaMemsetAsync(h->d_fz_status, 0, 4, cs) != cudaSuccess ||
         cudaStreamSynchronize(cs) != cudaSuccess) {
       set_error("fused-step set-up failed");
@@ -1215,6 +1215,9 @@ int ktune_search_create(ktune_space *s, ktune_model *m, const ktune_search_opts 
     if (N >= kFusedDefaultMin || (h->mode == 0 && !h->small))
       h->fused = !fotf && few && fused_blocks_per_sm(0) >= 1 ? 1 : fshape;
     h->fused_untimed = N < kFusedDefaultMin;
+    const bool shared = h->fused_untimed && h->mode == 0;
+    h->wait_grid = shared ? shared_grid(N, h->num_sms, true) : h->fused_grid;
+    h->async_grid = shared ? shared_grid(N, h->num_sms, false) : h->fused_grid;
   }
   *out = h;
   return KTUNE_OK;
@@ -1431,7 +1434,10 @@ static int enqueue_step(ktune_search *h, const float *counters, int k, int64_t *
     fa.words = h->d_fz_words;
     fa.terms = h->d_fz_terms;
     fa.mm_live = h->d_fz_mm;
-    fa.sync = h->d_fz_sync;
+    // (a grid's barrier counters count whole grids: one pair per grid size)
+    const bool waits = status_out != nullptr;
+    const int grid = waits ? h->wait_grid : h->async_grid;
+    fa.sync = h->d_fz_sync + (grid == h->fused_grid ? 0 : waits ? 2 : 4);
     fa.status = h->d_fz_status;
     fa.status_out = status_out;
     fa.cand = h->d_fz_cand;
@@ -1442,7 +1448,7 @@ static int enqueue_step(ktune_search *h, const float *counters, int k, int64_t *
     fa.st = sp;
     if (h->timing) CK(cudaEventRecord(h->ev[0], st));
     CK(launch_step_fused(fa, h->fused - 1, h->opts.select == KTUNE_SELECT_TOPK, h->model->D,
-                         h->fused_grid, st, h->mode == 2));
+                         grid, st, h->mode == 2));
     if (h->timing) CK(cudaEventRecord(h->ev[1], st));
   } else if (st != nullptr && h->use_graph) {
     TRY(launch_step_graph(h, sb, st));
@@ -1839,6 +1845,7 @@ int ktune_search_set_fused(ktune_search *h, int shape) {
   CK(cudaStreamSynchronize(h->last_stream));
   h->fused = shape;
   h->small = h->fused_untimed = false;
+  h->wait_grid = h->async_grid = h->fused_grid;
   return KTUNE_OK;
 }
 

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "ktune.h"
+#include "plan.h"
 
 namespace ktune {
 
@@ -592,13 +593,14 @@ struct ktune_search {
   int fused = 0;
   bool small = false;                  // steps as one CTA (k_small.cu), until a shape is asked for
   bool fused_untimed = false;          // `fused` holds only while no per-kernel times are asked for
-  int fused_grid = 0;
+  int fused_grid = 0;                  // every SM
+  int wait_grid = 0, async_grid = 0;   // the default's, for ktune_step and ktune_step_device
   bool last_fused = false;
   uint32_t *d_fz_words = nullptr;      // [K][L] node words
   float *d_fz_terms = nullptr;         // [K][L] the step's per-leaf summands
   uint64_t *d_fz_phase = nullptr;      // [8] phase time stamps (timing enabled)
   int *d_fz_mm = nullptr;              // [2] live min / max
-  unsigned long long *d_fz_sync = nullptr;
+  unsigned long long *d_fz_sync = nullptr;   // [3][2] barrier counters: of fused_grid, wait_grid, async_grid
   int *d_fz_status = nullptr;
   uint64_t *d_fz_cand = nullptr;       // [grid][KTUNE_MAX_K]
   uint32_t *d_fz_list = nullptr;       // on-the-fly spaces: TS's one-word digits, rebuilt each step
