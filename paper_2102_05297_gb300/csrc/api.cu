@@ -1895,49 +1895,32 @@ struct BatchVariant {
 const BatchVariant kBatchVariants[] = {{0, 1}, {0, 4}, {1, 1}, {2, 1}, {2, 4}, {3, 1}, {4, 1}, {4, 4}};
 constexpr int kNumBatchVariants = sizeof(kBatchVariants) / sizeof(kBatchVariants[0]);
 
-// Work items of the batch: every search's space (ordinals, or raw tiles when on
-// the fly), one after the other, cut into SMs * items_per_cta bins of equal cost;
-// a bin that ends inside a search leaves the rest to the next one, so a CTA's
-// bin is a run of neighbouring items.  A piece costs its units and, as it has to
-// stage the search's trees, what about kPieceCost of them would.  (Pieces of
-// total / SMs units of every search on its own gave 32 searches 185 items for
-// 152 CTAs, so that some CTAs had two: 191 us of score kernel, now 173; see
-// k_bscore's bins.)
+// Work items of the batch (cut_bins): SMs * items_per_cta bins, of the score kernel's
+// chunks, or of raw tiles on the fly (a warp each).  To stage a search's trees costs
+// about what kPieceCost configurations do.
 constexpr int64_t kPieceCost = 1024;
 int batch_items(ktune_batch *b) {
-  std::vector<ItemDev> items;
+  std::vector<int64_t> units;
+  for (ktune_search *h : b->s)     // (those scored by the MLP kernels have no tree-walk items)
+    units.push_back(h->model->kind == 2 ? 0 : b->mode == 2 ? h->space->n_tiles : h->space->n_valid);
+  const int64_t chunk =
+      b->mode == 2 ? 1 : (int64_t)bscore_variant_threads(b->variant) * bscore_variant_cpt(b->variant);
+  std::vector<ktune::Cut> cuts;
   std::vector<int> first;
-  const int bins = b->num_sms * b->items_per_cta;
-  const int64_t piece = b->mode == 2 ? 1 : kPieceCost;
-  int64_t total = 0;
-  for (ktune_search *h : b->s)
-    if (h->model->kind != 2) total += (b->mode == 2 ? h->space->n_tiles : h->space->n_valid) + piece;
-  // (every bin may start a piece and leave up to a piece's cost unused)
-  const int64_t target = std::max<int64_t>(2 * piece, (total + bins - 1) / bins + 2 * piece);
-  int64_t room = 0;    // left in the current bin
-  for (size_t i = 0; i < b->s.size(); ++i) {
-    ktune_search *h = b->s[i];
+  ktune::cut_bins(units, b->num_sms * b->items_per_cta, chunk, b->mode == 2 ? 1 : kPieceCost, &cuts, &first);
+  std::vector<ItemDev> items;
+  for (size_t i = 0, at = 0; i < b->s.size(); ++i) {
     b->sdh[i].item_begin = (int64_t)items.size();
-    if (h->model->kind != 2) {   // (those scored by the MLP kernels have no tree-walk items)
-      const int64_t units = b->mode == 2 ? h->space->n_tiles : h->space->n_valid;
-      for (int64_t lo = 0; lo < units;) {
-        if (room <= piece) {
-          first.push_back((int)items.size());
-          room = target;
-        }
-        ItemDev it{};
-        it.search = (int)i;
-        it.lo = lo;
-        it.hi = std::min(units, lo + room - piece);
-        items.push_back(it);
-        room -= it.hi - lo + piece;
-        lo = it.hi;
-      }
+    for (; at < cuts.size() && cuts[at].search == (int)i; ++at) {
+      ItemDev it{};
+      it.search = (int)i;
+      it.lo = cuts[at].lo;
+      it.hi = cuts[at].hi;
+      items.push_back(it);
     }
     b->sdh[i].item_end = (int64_t)items.size();
   }
-  b->n_bins = (int)first.size();
-  first.push_back((int)items.size());
+  b->n_bins = (int)first.size() - 1;
   b->n_items = (int)items.size();
   b->grid = std::min<int>(b->n_bins, b->num_sms);
   cudaFree(b->d_first);

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <vector>
 
 namespace ktune {
 
@@ -33,6 +34,49 @@ inline int shared_grid(int64_t N, int sms, bool waits) {
   const int64_t g = waits ? (by_1024 <= sms ? by_1024 : std::min<int64_t>((N + 1535) / 1536, sms - sms / 8))
                           : std::max(std::min<int64_t>(by_1024, std::max(1, sms / 4)), (N + 4095) / 4096);
   return (int)std::min<int64_t>(g, sms);
+}
+
+// A batch's searches, of units[i] configurations (raw tiles on the fly), cut into work
+// items, item after item dealt into at most `bins` bins (a CTA's share): bin b holds
+// items first[b] .. first[b + 1).  A CTA takes a whole chunk of configurations in the
+// time of one, so items are whole chunks but for a search's last, and an item costs
+// its chunks and `piece` more, as it stages its search's trees.  The bins' common size
+// is the smallest with which they suffice: searches that need no cutting have a bin
+// each while there are bins.  us per batched step, depth-12 trees for 32 counters, 152
+// SMs (pieces of total / SMs configurations of each search, dealt out in turn / even
+// bins with room to spare / here): 64 searches of 500 configurations 281 / 286 / 268,
+// 32 each of 40,960 and 500 332 / 354 / 299, 8 each of 196,608, 3,600, 500 and 16,384
+// 245 / 284 / 199.
+struct Cut {
+  int search;
+  int64_t lo, hi;
+};
+inline void cut_bins(const std::vector<int64_t> &units, int bins, int64_t chunk, int64_t piece,
+                     std::vector<Cut> *items, std::vector<int> *first) {
+  int64_t total = 0;
+  for (int64_t u : units)
+    if (u > 0) total += (u + chunk - 1) / chunk * chunk + piece;
+  auto fill = [&](int64_t size) {
+    int64_t room = 0;
+    items->clear();
+    first->clear();
+    for (size_t i = 0; i < units.size(); ++i)
+      for (int64_t lo = 0; lo < units[i];) {
+        if (room < piece + chunk) {
+          first->push_back((int)items->size());
+          room = size;
+        }
+        const int64_t n = std::min((room - piece) / chunk, (units[i] - lo + chunk - 1) / chunk);
+        const int64_t hi = std::min(units[i], lo + n * chunk);
+        items->push_back({(int)i, lo, hi});
+        room -= piece + n * chunk;
+        lo = hi;
+      }
+    return (int)first->size();
+  };
+  int64_t size = std::max(piece + chunk, (total + bins - 1) / bins);
+  while (fill(size) > bins) size += piece;
+  first->push_back((int)items->size());
 }
 
 }  // namespace ktune
