@@ -1199,8 +1199,8 @@ int ktune_search_create(ktune_space *s, ktune_model *m, const ktune_search_opts 
       set_error("fused-step set-up failed");
       return fail(KTUNE_ECUDA);
     }
-    // Up to kSmallMax configurations (weighted draws) one CTA does the step, while
-    // no per-kernel times are asked for; above, one persistent kernel.  With at most
+    // Over the smallest spaces (small_step) one CTA does the step, while no per-kernel
+    // times are asked for; else one persistent kernel.  With at most
     // 4,096 configurations per CTA, one chunk of either shape, it has 512 threads,
     // whose warps walk only the configurations they have and whose barriers are
     // cheaper; from there on 1,024 threads hide more of the walks' latency.  us per
@@ -1209,8 +1209,10 @@ int ktune_search_create(ktune_space *s, ktune_model *m, const ktune_search_opts 
     // 53.1, 393,216 55.1 / 52.5 / 54.8, 589,824 - / 52.5 / 55.5, 983,040 - / 64.8 /
     // 65.8 (depth 8: 44.4 / 37.6 / -, 44.8 / 41.1 / 45.2, 45.1 / 46.6 / 47.4, - /
     // 48.4 / 47.3, - / 58.0 / 55.1); top-k, 40 counters: 163,840 71.1 / 47.7 / -,
-    // 589,824 - / 59.4 / 60.2, 983,040 - / 74.9 / 72.3.
-    h->small = h->mode == 0 && o->select == KTUNE_SELECT_SAMPLE && small_step_supported(N, m->D);
+    // 589,824 - / 59.4 / 60.2, 983,040 - / 74.9 / 72.3.  (The shapes cross a little
+    // below one full chunk with depth-8 trees and at two with depth-12 ones; on the
+    // wrong side of this line each loses 2% at most.)
+    h->small = h->mode == 0 && o->select == KTUNE_SELECT_SAMPLE && small_step(N, m->D);
     const bool few = N <= (int64_t)4096 * h->fused_grid;
     if (N >= kFusedDefaultMin || (h->mode == 0 && !h->small))
       h->fused = !fotf && few && fused_blocks_per_sm(0) >= 1 ? 1 : fshape;

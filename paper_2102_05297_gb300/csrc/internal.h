@@ -219,9 +219,7 @@ struct FusedArgs {
   uint32_t four;                  // 4, as a launch parameter (the walk's word-offset multiplier)
   StepDev st;
 };
-// The step of a small space as one CTA (k_small.cu).
-constexpr int64_t kSmallMax = 4096;
-bool small_step_supported(int64_t N, int D);
+// The step of a small space (small_step) as one CTA (k_small.cu).
 cudaError_t launch_step_small(const FusedArgs &fa, cudaStream_t st);
 int fused_shapes();
 int fused_blocks_per_sm(int shape);

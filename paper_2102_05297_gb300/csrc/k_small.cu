@@ -31,6 +31,7 @@ constexpr int kSmallThreads = 1024;
 constexpr int kSmallSmem = 200 * 1024;
 // per configuration: weight, score, digits; per thread: prefix sum
 constexpr int kSmallFixed = kSmallMax * 12 + kSmallThreads * 8;
+static_assert(kSmallFixed + 2 * (8 << 13) <= kSmallSmem, "two trees of depth 13");
 
 template <int CPT>
 __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const __grid_constant__ FusedArgs fa) {
@@ -282,9 +283,6 @@ cudaError_t launch_small_t(const FusedArgs &fa, cudaStream_t st) {
 }
 
 }  // namespace
-
-// At least one tree fits beside the configurations (depth 14: 128 KB a tree).
-bool small_step_supported(int64_t N, int D) { return N <= kSmallMax && kSmallFixed + (8 << D) <= kSmallSmem; }
 
 cudaError_t launch_step_small(const FusedArgs &fa, cudaStream_t st) {
   if (fa.sd.N <= kSmallThreads) return launch_small_t<1>(fa, st);

@@ -9,6 +9,19 @@
 
 namespace ktune {
 
+// Weighted-draw steps over materialised one-word spaces that one CTA does by default: up
+// to kSmallMax configurations, four per thread, while the staged trees come in few
+// groups (147 KB: four of depth 12, two of depth 13, one of depth 14; a group is a round
+// trip and three barriers, and every tree's summands are made by this CTA alone).  us
+// per step, 32 counters (one CTA / the persistent kernel / four kernels), 1,024, 2,048,
+// 3,072 and 4,096 configurations:
+//   depth  8   23.8 / 35.3 / 41.2   25.0 / 34.8 / 41.2   28.4 / 34.2 / 40.6   30.3 / 38.1 / 43.7
+//   depth 12   33.5 / 41.8 / 48.4   34.9 / 40.1 / 49.5   39.4 / 40.8 / 51.3   40.0 / 38.6 / 48.9
+//   depth 13   40.7 / 41.8 / 48.0   46.2 / 46.9 / 54.4   51.1 / 46.9 / 55.3   54.2 / 47.6 / 56.1
+//   depth 14   64.5 / 61.1 / 66.1   67.5 / 60.3 / 68.6   74.5 / 62.0 / 69.4   75.0 / 58.5 / 66.1
+constexpr int64_t kSmallMax = 4096;
+inline bool small_step(int64_t N, int D) { return N <= kSmallMax && D <= (N <= 2048 ? 13 : 12); }
+
 // CTAs of the persistent step of a search over N configurations, by default and below
 // 2^18 of them (larger spaces fill the GPU in any case).  The kernel holds an SM per
 // CTA for as long as its chain of latencies lasts, so with a CTA on every SM the steps

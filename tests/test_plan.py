@@ -9,6 +9,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 WRAP = """
 #include "plan.h"
 extern "C" int grid(long long N, int sms, int waits) { return ktune::shared_grid(N, sms, waits != 0); }
+extern "C" int small_step(long long N, int D) { return ktune::small_step(N, D); }
 extern "C" void bins(const long long *units, int n, int bins, long long chunk, long long piece, long long *out,
                      int *first, int *counts) {
   std::vector<ktune::Cut> c;
@@ -93,3 +94,10 @@ def test_bins_of_a_batch(plan, units, bins, chunk, piece):
     assert max(loads) <= max(chunk + piece, even + chunk + 2 * piece)
     if sum(-(-u // chunk) for u in units) <= bins:
         assert max(loads) == chunk + piece
+
+
+def test_one_cta_only_where_trees_come_in_few_groups(plan):
+    for D in range(0, 13):
+        assert [plan.small_step(n, D) for n in (1, 2048, 2049, 4096, 4097)] == [1, 1, 1, 1, 0]
+    assert [plan.small_step(n, 13) for n in (1, 2048, 2049, 4096)] == [1, 1, 0, 0]
+    assert not any(plan.small_step(n, 14) for n in (1, 1024, 2048, 4096))
