@@ -22,9 +22,9 @@
 // launches are scheduled while their predecessor drains (82 -> 77 us per step,
 // 16 steps of 4,096 rows; as 38 launches, one GEMM per layer and direction,
 // transposes, sums and one Adam per tensor, a step took 299 us).
-// Every wait on the tensor cores is bounded: on time-out the kernels record
-// KTUNE_ETIMEOUT, wait once more (bounded) for their MMAs in flight and go on
-// to their end with whatever was computed.
+// Every wait is bounded: on time-out the kernels record KTUNE_ETIMEOUT, wait once
+// more (bounded) for the copies and MMAs in flight and go on to their end with
+// whatever was computed.
 #include <float.h>
 #include <limits.h>
 
@@ -158,6 +158,13 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
   tc::fence_after();
   const uint32_t tmem = tmem_base, lanes = (uint32_t)((warp & 3) * 32) << 16;
   const bool lead = warp == 0 && tc::elect_one();
+  // A wait that has run out waits once more: what it waited for (a copy into this CTA, MMAs
+  // of its own) is not to arrive after the CTA has left.
+  auto wait = [&](uint64_t *bar, uint32_t phase) {
+    if (tc::mbar_wait(bar, phase, kTrainWait)) return true;
+    tc::mbar_wait(bar, phase, kTrainWait);
+    return false;
+  };
   uint32_t n_mma = 0, n_w[2] = {0u, 0u}, n_x = 0;     // phases passed; exchanges begun
 
   // Layer i of seven (forward 0..3, backward 4..6): D[dcol ..) = a * w^T over Kd columns,
@@ -166,8 +173,8 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
   auto layer = [&](int i, uint32_t a, int x, int Kd, int N, uint32_t dcol, const uint16_t *next, int next_bytes) {
     const int s = i & 1;
     if (warp == 0) {                 // the whole warp, so that descriptors live in uniform registers
-      ok = tc::mbar_wait(&w_full[s], n_w[s] & 1u, kTrainWait) && ok;
-      if (x >= 0) ok = tc::mbar_wait(&a_full[x & 1], (uint32_t)(x >> 1) & 1u, kTrainWait) && ok;
+      ok = wait(&w_full[s], n_w[s] & 1u) && ok;
+      if (x >= 0) ok = wait(&a_full[x & 1], (uint32_t)(x >> 1) & 1u) && ok;
       tc::fence_async_smem();
       tc::fence_after();
       const uint32_t idesc = tc::idesc_bf16(128, N);
@@ -182,10 +189,8 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
       __syncwarp();
     }
     ++n_w[s];
-    bool w_ok = tc::mbar_wait(&mma, n_mma & 1u, kTrainWait);
-    if (!w_ok) w_ok = tc::mbar_wait(&mma, n_mma & 1u, kTrainWait) && false;   // the MMAs still in flight
+    ok = wait(&mma, n_mma & 1u) && ok;
     ++n_mma;
-    ok = ok && w_ok;
     tc::fence_after();
     if (next && threadIdx.x == 0) bulk_g2s(wb0 + (uint32_t)s * kWBuf, next, (uint32_t)next_bytes, &w_full[s]);
   };
@@ -325,7 +330,7 @@ __global__ void __cluster_dims__(kSplitN, 1, 1) __launch_bounds__(kRowThreads, 1
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i) h[i] = bf2(v[2 * i], v[2 * i + 1]);
-    if (l == 2) ok = tc::mbar_wait(&freed, 0u, kTrainWait) && ok;
+    if (l == 2) ok = wait(&freed, 0u) && ok;
     if (l > 0) share(act0 + (uint32_t)((l & 1) ^ 1) * kActBuf, h);
     else tc::fence_before();
     store_t(td.gzt[l], h);
