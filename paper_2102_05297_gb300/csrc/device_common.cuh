@@ -73,12 +73,6 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
                "l"(gmem_src)
                : "memory");
 }
-__device__ __forceinline__ void cp_async8(void *smem_dst, const void *gmem_src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
-                   (uint32_t)__cvta_generic_to_shared(smem_dst)),
-               "l"(gmem_src)
-               : "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // Groups of copies: commit the copies issued so far as one group; wait until
 // at most N of this thread's groups are still pending.

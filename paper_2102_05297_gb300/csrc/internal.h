@@ -316,7 +316,7 @@ constexpr int kMlpMaxSplits = 64;       // split-K slices of the weight-gradient
 // layer's rows padded to a multiple of 32 (a pair MMA's N)
 constexpr int kMlpChunkK = 64;
 __host__ __device__ inline int mlp_chunk_k(int l) { return l == 3 ? kMlpHidden : kMlpChunkK; }
-__host__ __device__ inline int mlp_n4(int K) { return (K + 31) & ~31; }
+__host__ __device__ constexpr int mlp_n4(int K) { return (K + 31) & ~31; }
 
 // The network as the fused forward kernel reads it (all device pointers).
 struct MlpDev {

@@ -24,22 +24,6 @@ namespace {
 
 constexpr uint64_t kWaitLimit = 1000000000ull;   // 1 s per tensor-core wait
 
-// Rows [0, rows) x columns [k0, k0 + kc) of a bf16 row-major matrix into
-// shared memory in the core-matrix layout with KC = kc, by asynchronous
-// 16-byte copies; rows >= valid are 0.  kc is a multiple of 16; ld a multiple
-// of 8; src 16-byte aligned.
-__device__ __forceinline__ void load_tile(uint8_t *dst, const uint16_t *src, int ld, int rows,
-                                          int valid, int k0, int kc) {
-  const int per_row = kc >> 3;
-  const int pieces = rows * per_row;
-  for (int p = threadIdx.x; p < pieces; p += blockDim.x) {
-    const int r = p / per_row, kb = p - r * per_row;
-    uint8_t *d = dst + tc::core_off(r, kb * 8, kc);
-    if (r < valid) cp_async16(d, src + (size_t)r * ld + k0 + kb * 8);
-    else *reinterpret_cast<uint4 *>(d) = make_uint4(0, 0, 0, 0);
-  }
-}
-
 // MMAs over one K chunk: D (+)= A[:, a_k0 : a_k0 + kc] * B^T, A stored with
 // KC = kcA (128 rows), the B chunk with KC = kc (N rows).
 __device__ __forceinline__ void issue_chunk(uint32_t tmem, const uint8_t *sA, int kcA, int a_k0,
@@ -88,8 +72,8 @@ __global__ void __launch_bounds__(128, 1)
   auto stage_b = [&](int c) { return sm + (c & 1) * kGemmStage + 16384; };
   auto issue = [&](int c) {
     const int k0 = c * 64, kc = K - k0 < 64 ? K - k0 : 64;
-    load_tile(stage_a(c), A + (size_t)m0 * lda, lda, 128, M - m0, k0, kc);
-    load_tile(stage_b(c), B + (size_t)n0 * ldb, ldb, Nt, Nt, k0, kc);
+    tc::load_tile(stage_a(c), A + (size_t)m0 * lda, lda, 128, M - m0, k0, kc);
+    tc::load_tile(stage_b(c), B + (size_t)n0 * ldb, ldb, Nt, Nt, k0, kc);
     cp_async_commit();
   };
   if (c_lo < c_hi) issue(c_lo);

@@ -20,7 +20,7 @@
 //                cores (a proxy fence) and tells the even CTA.
 // The MMAs of one tile run during the epilogue of the other.
 //
-// What bounds it: the FMA pipe in the epilogue (14 paired and 4 single
+// What bounds it: the FMA pipe in the epilogue (12 paired and 4 single
 // instructions for two activations, 28 cycles of the pipe; 3.6k cycles per tile
 // and layer, 4.4k measured) and, tile by tile, the chain from a tile's last
 // stored activation to its next accumulator (5.2k cycles: both CTAs' hand-over
@@ -92,6 +92,11 @@ struct alignas(16) PairShared {
 static_assert(offsetof(PairShared, bias) % 16 == 0, "bias is read as float4");
 constexpr int kPairSmem = 2 * kActBytes + kSlots * kSlotBytes + (int)sizeof(PairShared);
 static_assert(kPairSmem <= 227 * 1024, "shared memory of one CTA");
+// the MMAs of a layer wait for all of its chunks, and only they free the ring's slots
+static_assert((kMlpMaxF + kMlpChunkK - 1) / kMlpChunkK <= kSlots && kMlpHidden / kMlpChunkK <= kSlots,
+              "a layer's chunks fit the ring");
+static_assert(mlp_n4(KTUNE_MAX_COUNTERS) / 2 * kMlpHidden * 2 <= kSlotBytes, "the output layer's half is one slot");
+static_assert(kMaxGroups8 <= 32, "a lane per feature group");
 
 __device__ __forceinline__ void ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(

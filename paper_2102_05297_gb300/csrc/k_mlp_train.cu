@@ -4,19 +4,21 @@
 //                  three hidden layers, the output layer with the loss and its
 //                  gradient, and the three backward layers -- for 128 rows per
 //                  cluster of four CTAs.  CTA r computes columns [64 r, 64 r + 64)
-//                  of every hidden layer (tcgen05, M = 128, N = 64) and stores
-//                  its bfloat16 activations into all four CTAs' operand buffers
-//                  (distributed shared memory); pre-activations stay in tensor
-//                  memory as accumulators (z = accumulator + bias again in the
-//                  backward pass), so no layer reads or writes memory but for
-//                  the transposes that the weight gradients need;
+//                  of every hidden layer (tcgen05, M = 128, N = 64), stores its
+//                  bfloat16 activations into its block of the operand buffer and
+//                  sends the block to the other three by bulk copies between
+//                  their shared memories, each counted in by an mbarrier of its
+//                  reader (no cluster barrier between layers); pre-activations
+//                  stay in tensor memory as accumulators (z = accumulator + bias
+//                  again in the backward pass), so no layer reads or writes
+//                  memory but for the transposes that the weight gradients need;
 //   k_train_wgrad  the four weight gradients, whose reduction runs over the
 //                  batch, split over up to 64 slices of rows, each slice's tile
 //                  into a workspace, and the bias gradients' row-block sums;
 //   k_train_update the slices summed in a fixed order, and Adam.
 // What bounds it: latency.  The step's arithmetic is 0.4 GFLOP x 9 (about 2 us of
 // tensor work at 4,096 rows); k_train_rows is a chain of seven layers, each an
-// MMA, an epilogue of erff / expf and a cluster barrier.  4,096 rows (128
+// MMA, an epilogue of erff / expf and an exchange of blocks.  4,096 rows (128
 // CTAs): k_train_rows 36 us, k_train_wgrad 18, k_train_update 6; the update of
 // one step and the rows of the next do not overlap (the weights), the other two
 // launches are scheduled while their predecessor drains (82 -> 77 us per step,
@@ -354,19 +356,6 @@ constexpr int kWgStage = 2 * kWgTile * 64 * 2;   // both operands' 64 columns of
 constexpr int kWgSmem = 2 * kWgStage;            // three CTAs per SM
 constexpr int kColRows = 256;                    // rows per block of the bias gradients' sums
 
-// Rows [0, rows) x columns [k0, k0 + kc) into core matrices with KC = kc by
-// asynchronous copies; rows >= valid are 0.
-__device__ __forceinline__ void load_tile(uint8_t *dst, const uint16_t *src, int ld, int rows, int valid,
-                                          int k0, int kc) {
-  const int per_row = kc >> 3, pieces = rows * per_row;
-  for (int p = threadIdx.x; p < pieces; p += blockDim.x) {
-    const int r = p / per_row, kb = p - r * per_row;
-    uint8_t *d = dst + tc::core_off(r, kb * 8, kc);
-    if (r < valid) cp_async16(d, src + (size_t)r * ld + k0 + kb * 8);
-    else *reinterpret_cast<uint4 *>(d) = make_uint4(0, 0, 0, 0);
-  }
-}
-
 // Blocks below wg_blocks: slice z of one 128 x 128 tile of a weight gradient
 // (G^T X over the slice's rows) into the workspace.  The blocks behind them: one
 // (32 columns, 256 rows) block of a bias gradient, in the order of a 32-row
@@ -421,8 +410,8 @@ __global__ void __launch_bounds__(kWgThreads) k_train_wgrad(const __grid_constan
   auto issue = [&](int c) {
     const int k0 = c * 64, kc = min(64, B - k0);
     uint8_t *s = sm + (c & 1) * kWgStage;
-    load_tile(s, A, B, kWgTile, M - m0, k0, kc);
-    load_tile(s + kWgStage / 2, X, B, Nt, Nt, k0, kc);
+    tc::load_tile(s, A, B, kWgTile, M - m0, k0, kc);
+    tc::load_tile(s + kWgStage / 2, X, B, Nt, Nt, k0, kc);
     cp_async_commit();
   };
   auto done = [&]() {
@@ -432,7 +421,7 @@ __global__ void __launch_bounds__(kWgThreads) k_train_wgrad(const __grid_constan
     ok = ok && w;
     tc::fence_after();
   };
-  if (lo < hi) issue(lo);
+  issue(lo);                  // (never more slices than chunks: none is empty)
   for (int c = lo; c < hi; ++c) {
     // the MMAs of chunk c - 1 read the stage that chunk c + 1 is copied into
     if (c > lo) {
@@ -458,18 +447,12 @@ __global__ void __launch_bounds__(kWgThreads) k_train_wgrad(const __grid_constan
       tc::mma_commit(&mbar);
     }
   }
-  if (lo < hi) done();
-  // slices of fewer rows than 64 x splits may be empty: zeros
+  done();
   const int row = m0 + (warp & 3) * 32 + lane;
   float *out = wd.ws[p] + (size_t)z * M * N + (size_t)c0 * M + row;
   for (int c = 16 * (warp >> 2); c < Nt; c += 32) {
     float v[16];
-    if (lo < hi) {
-      tc::tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + c, v);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = 0.0f;
-    }
+    tc::tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + c, v);
     if (row < M)
 #pragma unroll
       for (int i = 0; i < 16; ++i) out[(size_t)(c + i) * M] = v[i];

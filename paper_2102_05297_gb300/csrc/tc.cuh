@@ -13,6 +13,8 @@
 
 #include <stdint.h>
 
+#include "device_common.cuh"
+
 namespace ktune {
 namespace tc {
 
@@ -153,6 +155,22 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Rows [0, rows) x columns [k0, k0 + kc) of a bf16 row-major matrix into
+// shared memory in the core-matrix layout with KC = kc, by asynchronous
+// 16-byte copies; rows >= valid are 0.  kc is a multiple of 16; ld a multiple
+// of 8; src 16-byte aligned.
+__device__ __forceinline__ void load_tile(uint8_t *dst, const uint16_t *src, int ld, int rows,
+                                          int valid, int k0, int kc) {
+  const int per_row = kc >> 3;
+  const int pieces = rows * per_row;
+  for (int p = threadIdx.x; p < pieces; p += blockDim.x) {
+    const int r = p / per_row, kb = p - r * per_row;
+    uint8_t *d = dst + tc::core_off(r, kb * 8, kc);
+    if (r < valid) cp_async16(d, src + (size_t)r * ld + k0 + kb * 8);
+    else *reinterpret_cast<uint4 *>(d) = make_uint4(0, 0, 0, 0);
+  }
 }
 
 // ---- CTA pairs (cta_group::2): two CTAs of a cluster on one 256-row tile ----
