@@ -537,7 +537,6 @@ int ktune_space_create(const ktune_space_desc *d, int flags, void *stream, ktune
                                   cudaMemcpyDeviceToHost, cs);
   if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
   if (e == cudaSuccess) e = cudaGetLastError();
-  drop(d_count);
   if (e == cudaSuccess && flags == KTUNE_MATERIALISE) {
     WordArgs wa{};
     for (int j = 0; j < s->sa.P; ++j) wa.pos[j] = s->pos[j];
@@ -553,6 +552,7 @@ int ktune_space_create(const ktune_space_desc *d, int flags, void *stream, ktune
     }
     if (rc) {
       drop(d_masks);
+      drop(d_count);
       return cleanup(rc);
     }
     launch_enum_write(s->sa, s->d_groups, s->d_table, d_masks, s->n_tiles, s->d_tile_offset, s->d_packed,
@@ -561,6 +561,7 @@ int ktune_space_create(const ktune_space_desc *d, int flags, void *stream, ktune
     if (e == cudaSuccess) e = cudaGetLastError();
   }
   drop(d_masks);
+  drop(d_count);
   if (e != cudaSuccess) {
     set_error(std::string("enumeration: ") + cudaGetErrorString(e));
     return cleanup(KTUNE_ECUDA);
