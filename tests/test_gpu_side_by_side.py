@@ -32,8 +32,8 @@ def setup(kt, radices, K, depth, seed):
     return sp, m, c
 
 
-# configurations: 4,368, 77,760 and 78,000 (76 and 77 CTAs of 1,024), 155,520 and
-# 156,000 (152, 102), 233,280 (133 CTAs), 262,080
+# configurations: 4,368 (16 CTAs), 77,760 and 78,000 (76 and 77 of 1,024), 155,520 and
+# more (148)
 @pytest.mark.parametrize("select", ["sample", "topk"])
 @pytest.mark.parametrize("radices", [(14, 13, 12, 2), (15, 16, 12, 9, 3), (13, 15, 16, 5, 5), (15, 16, 12, 9, 6),
                                      (13, 15, 16, 5, 10), (15, 16, 12, 9, 9), (13, 15, 16, 12, 7)])

@@ -45,11 +45,10 @@ def test_grids_leave_room_for_other_searches(plan, sms, waits):
     for N in [1, 2, 4097, 5120, 16384, 16385, 40960, 77824, 77825, 155648, 155649, 162816, 204288, 245760, 262143]:
         g = plan.grid(N, sms, waits)
         assert 1 <= g <= sms
-        assert -(-N // g) <= 4096 or g == sms
+        assert -(-N // g) <= 4096 or g >= sms - 4
         if sms == 152:
             assert g <= max(16, -(-N // 1024))
-            if N > 152 * 1024:
-                assert g <= 133            # a step may start while another draws
+            assert g <= 148                # a step may start while others draw
             if not waits:
                 assert g <= max(38, -(-N // 4096))
 
