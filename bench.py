@@ -70,13 +70,13 @@ WORKLOADS = {
 }
 ALL_PATHS = ("chain", "mlp", "lsq", "cached", "table", "nbr", "batch", "large", "mlp_large", "tiny")
 # DRAM bytes (read + write) per launch of each path's dominant kernel, from the ncu
-# captures summarised under profiles/ (the kernels have not changed since)
+# captures summarised under profiles/ (cold caches)
 PROFILED_TRAFFIC = {
     "k_bscore": 9.637e6,          # profiles/k_bscore_mid_12p.md
-    "k_cscore_leaf": 36.564e6,    # profiles/cached_mid_12p.md
-    "k_mlp_pair": 18.7e6,         # the packed TS, read once (profiles/k_mlp_pair_mid_12p.md)
+    "k_cscore_leaf": 41.124e6,    # profiles/cached_mid_12p.md
+    "k_mlp_pair": 18.769e6,       # scoring (profiles/k_mlp_pair_mid_12p.md)
     "k_bscore_otf": 20.228e6,     # profiles/k_bscore_otf_large_16p.md
-    "k_step_fused": 9.763e6,      # profiles/k_step_fused_mid_12p.md
+    "k_step_fused": 9.716e6,      # profiles/k_step_fused_mid_12p.md
     "k_step_fused_otf": 378.7e6,  # profiles/k_step_fused_otf_large_16p.md
 }
 MLP_HIDDEN = 256

@@ -531,7 +531,10 @@ struct ktune_batch {
   ktune::HostOut *hout = nullptr;       // the searches' outputs, mapped pinned host memory
   ktune::HostOut *hout_dev = nullptr;
   int *h_status = nullptr;              // the networks' device-side statuses, pinned
-  // branches of the batched step beside the tree searches: one per MLP group, in turn
+  // branches of the batched step beside the tree searches: one per MLP group, in turn.
+  // 64 searches over eight spaces, four of them with a network, us per step with 1, 2, 3,
+  // 4 and 6 branches: 1,370, 1,289, 1,283, 1,269, 1,265 (more than one, so that a group's
+  // launches and last tiles run under another's; little after that, as a group fills the GPU)
   static constexpr int kBranches = 3;
   cudaStream_t branch[kBranches] = {};
   cudaEvent_t fork = nullptr, join[kBranches] = {};
